@@ -314,8 +314,15 @@ vp_status vp::validate(const vp_params *p, const vp_integrand *f, Member &mb) {
         mb.prm32.push_back((float)std::log2(1.0 / (s2pi * 10.0 * sy)));
         mb.prm32.push_back((float)(L2E / (2.0 * pw * pw)));
         mb.prm32.push_back((float)(lref * L2E));
-        for (int i = 0; i < np; ++i) mb.prm32.push_back((float)q[6 + i]);
-        for (int i = 0; i < np * P; ++i) mb.prm32.push_back((float)q[6 + np + i]);
+        const int stride = (1 + P + 3) & ~3;  // {y, A[0..P-1], pad} per point
+        mb.prm32.push_back((float)stride);
+        mb.prm32.resize(kPostHead, 0.0f);
+        for (int g = 0; g < G; ++g)  // group by group: the points of weight g
+            for (int i = g; i < np; i += G) {
+                mb.prm32.push_back((float)q[6 + i]);
+                for (int m = 0; m < stride - 1; ++m)
+                    mb.prm32.push_back(m < P ? (float)q[6 + np + i * P + m] : 0.0f);
+            }
     } else {
         // per peak {a, k, 0, 0, c[D], pad}: a multiple of 4 floats
         const int K = (int)q[0];

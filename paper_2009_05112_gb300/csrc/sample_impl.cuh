@@ -65,7 +65,9 @@ template <> struct Real<false> { typedef float T; };
 //  BALL     per peak {a, r^2, 0, 0, c[D], pad}          f = sum a [|x-c|^2 < r^2]
 //  EXPNORM  per peak {a, s log2(e), 0, 0, c[D], pad}    f = sum a 2^(-k |x-c|)
 //           (peaks padded to a multiple of 4 floats for 16-byte shared loads)
-//  POSTERIOR {n, P, G, kN, kW, lcN, lcW, kprior, logref2, y[n], A[n][P]} in log2 units
+//  POSTERIOR {n, P, G, kN, kW, lcN, lcW, kprior, logref2, stride, 0, 0}, then the points
+//           group by group (0, G, 2G, ..., 1, G + 1, ...), each {y, A[0..P-1], pad} on
+//           `stride` floats (a multiple of 4); in log2 units
 // ---------------------------------------------------------------------------
 template <int DMAX>
 __device__ __forceinline__ double f_peaks64(int kind, const double *p, int K, int dim,
@@ -185,35 +187,60 @@ __device__ __forceinline__ double f_post64(const double *p, int dim, const doubl
 }
 
 // FP32: the points are visited group by group (points g, g + G, g + 2G, ...
-// share the weight w_g), so that each w_g is read from a fixed register.
+// share the weight w_g), so that each w_g is read from a fixed register; the
+// constants hold them in that order, so the loop walks one pointer.
 // Returns log2 f: a posterior's values span hundreds of binary orders below
 // its maximum (a sharp 21-parameter one integrates to ~1e-28), far beyond the
 // FP32 range, so f is formed by the caller as a mantissa and an exponent.
-template <int DMAX>
-__device__ __forceinline__ float f_post32_log2(const float *p, int dim, const float (&x)[DMAX]) {
-    const int n = (int)p[0], npar = (int)p[1], ngrp = (int)p[2];
-    const float kN = p[3], kW = p[4], lcN = p[5], lcW = p[6], kpr = p[7], lref = p[8];
-    const float *y = p + 9;
-    const float *A = p + 9 + n;
+// Bound: the three MUFU operations of a point (6 cycles of an SM per warp and
+// point).  A line (P = 2) reads a point as one 16-byte shared load and takes
+// two multiply-adds; testing every m < DMAX against P, as the general form
+// once did here too, cost ~100 cycles per warp and point at D = 21.
+template <int DMAX, bool LINE>
+__device__ __forceinline__ float post32_points(const float *p, int n, int npar, int ngrp,
+                                               const float (&x)[DMAX]) {
+    const float kN = p[3], kW = p[4], lcN = p[5], lcW = p[6];
+    const int stride = LINE ? 4 : (int)p[9];
+    const float *q = p + kPostHead;
     float acc = 0.0f;
 #pragma unroll
     for (int mu = 1; mu < DMAX; ++mu) {
-        if (mu < npar || mu >= npar + ngrp) continue;
+        if (LINE ? mu < 2 : mu < npar) continue;
+        if (mu >= npar + ngrp) break;
         const float w = x[mu];
-        const float lw1 = lg2_approx(1.0f - w), lw = lg2_approx(w);
-        for (int i = mu - npar; i < n; i += ngrp) {
-            const float *a = A + i * npar;
-            float model = 0.0f;
+        const float cN = lcN + lg2_approx(1.0f - w), cW = lcW + lg2_approx(w);
+#pragma unroll(DMAX > 4 ? 1 : 4)
+        for (int i = mu - npar; i < n; i += ngrp, q += stride) {
+            float y, model;
+            if (LINE) {
+                const float4 v = *(const float4 *)q;
+                y = v.x;
+                model = fmaf(v.z, x[1], v.y * x[0]);
+            } else {
+                y = q[0];
+                model = 0.0f;
 #pragma unroll
-            for (int m = 0; m < DMAX; ++m)
-                if (m < npar) model = fmaf(a[m], x[m], model);
-            const float r = y[i] - model;
+                for (int m = 0; m < DMAX; ++m) {
+                    if (m >= npar) break;
+                    model = fmaf(q[1 + m], x[m], model);
+                }
+            }
+            const float r = y - model;
             const float r2 = r * r;
-            const float nar = ex2_approx(fmaf(-kN, r2, lcN + lw1));
-            const float wid = ex2_approx(fmaf(-kW, r2, lcW + lw));
+            const float nar = ex2_approx(fmaf(-kN, r2, cN));
+            const float wid = ex2_approx(fmaf(-kW, r2, cW));
             acc += lg2_approx(nar + wid);
         }
     }
+    return acc;
+}
+
+template <int DMAX>
+__device__ __forceinline__ float f_post32_log2(const float *p, int dim, const float (&x)[DMAX]) {
+    const int n = (int)p[0], npar = (int)p[1], ngrp = (int)p[2];
+    const float kpr = p[7], lref = p[8];
+    const float acc = npar == 2 ? post32_points<DMAX, true>(p, n, 2, ngrp, x)
+                                : post32_points<DMAX, false>(p, n, npar, ngrp, x);
     float c2 = 0.0f;
 #pragma unroll
     for (int m = 0; m < DMAX; ++m)

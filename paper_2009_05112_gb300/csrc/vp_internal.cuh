@@ -21,6 +21,7 @@ constexpr int kSub = 4;            // CTAs of the allocation kernels per block o
 constexpr int kSubH = kTreeBlock / kSub;
 constexpr int kMaxPeaks = 64;
 constexpr int kMaxPoints = 256;
+constexpr int kPostHead = 12;      // floats before the points of a posterior's FP32 constants
 constexpr int kInvTab = 4096;      // table of 1/n, 1/(n(n-1)) and log2 n for small integers n
 constexpr int kInvTabWords = 4 * kInvTab;  // 32 bytes per n: 1/n, 1/(n(n-1)), log2 n (2 floats), pad
 // several integrals from the same samples (App. B): at most kMaxOut outputs, the

@@ -337,6 +337,13 @@ vp_status vp::validate(const vp_params *p, const vp_integrand *f, Member &mb) {
             mb.prm32.push_back(0.0f);
             for (int i = 0; i < D4; ++i) mb.prm32.push_back(i < D ? (float)pk[2 + i] : 0.0f);
         }
+        // FP64: 1/w^2 of every peak after the blob (0: out of range, the
+        // kernels divide instead)
+        for (int k = 0; k < K; ++k) {
+            const double w = q[2 + k * (2 + D)], w2 = w * w;
+            const bool in = w2 >= std::ldexp(1.0, -1000) && w2 <= std::ldexp(1.0, 1000);
+            mb.prm.push_back(in ? 1.0 / w2 : 0.0);
+        }
     }
     return VP_OK;
 }
@@ -599,6 +606,7 @@ void vp::fill_desc(const Member &mb, const double *d_inv, Desc &d) {
     }
     div_magic((uint32_t)mb.n_st, &d.nst_magic, &d.nst_shift);
     d.uniform = mb.uniform ? 1u : 0u;
+    d.k_small = 1u;
     d.n_out = mb.n_out;
     d.d_weighted = mb.p.d_weighted;
     for (int k = 0; k < 2 * kMaxOut; ++k) d.mono[k] = k < (int)mb.mono.size() ? mb.mono[k] : -1;
@@ -616,6 +624,8 @@ void vp::fill_desc(const Member &mb, const double *d_inv, Desc &d) {
         div_magic(s, &d.strata.magic[mu], &d.strata.shift[mu]);
         d.strata.c32[mu] = (float)((double)G / (double)s);
         d.strata.nd[mu] = (double)s;
+        d.strata.rnd[mu] = 1.0 / (double)s;
+        if (s > (1u << 19)) d.k_small = 0u;
     }
     d.inv_tab = d_inv;
     d.edges = mbuf<double>(mb, B_EDGES);
@@ -766,6 +776,8 @@ static vp_status set_create(Set &s, int n, const vp_params *ps, const vp_integra
         L.ngD_m = d.ngD_m;
         L.ngD_e = d.ngD_e;
         L.nst = (double)d.n_st;
+        L.rnst = d.strata.rnd[0];
+        L.k_small = d.k_small != 0u;
         L.ng = (double)d.n_g;
         L.tab = d.tab;
         L.edges = d.edges;

@@ -69,9 +69,22 @@ template <> struct Real<false> { typedef float T; };
 //           group by group (0, G, 2G, ..., 1, G + 1, ...), each {y, A[0..P-1], pad} on
 //           `stride` floats (a multiple of 4); in log2 units
 // ---------------------------------------------------------------------------
+// a / b with rb = 1/b rounded to nearest (0: b outside [2^-1000, 2^1000], a
+// division): the quotient times rb corrected once by its exact residual, the
+// correctly rounded result but for quotients within 2^-51 units in the last
+// place of a midpoint.  An overflowing or NaN quotient passes unchanged.
+__device__ __forceinline__ double ratio64(double a, double b, double rb) {
+    if (rb == 0.0) return __ddiv_rn(a, b);
+    const double q = __dmul_rn(a, rb);
+    const double c = __fma_rn(__fma_rn(-b, q, a), rb, q);
+    return (__double2hiint(q) & 0x7ff00000) == 0x7ff00000 ? q : c;
+}
+
+// (p: the blob after its peak count; after the K peaks, 1/w^2 of each, see ratio64)
 template <int DMAX>
 __device__ __forceinline__ double f_peaks64(int kind, const double *p, int K, int dim,
                                             const double (&x)[DMAX]) {
+    const double *rw = p + K * (2 + dim);
     double f = 0.0;
     for (int k = 0; k < K; ++k) {
         const double a = p[0], w = p[1];
@@ -84,7 +97,7 @@ __device__ __forceinline__ double f_peaks64(int kind, const double *p, int K, in
                 r2 = __dadd_rn(r2, __dmul_rn(dx, dx));
             }
         }
-        if (kind == VP_GAUSS) f += a * exp(__ddiv_rn(-r2, __dmul_rn(w, w)));
+        if (kind == VP_GAUSS) f += a * exp(ratio64(-r2, __dmul_rn(w, w), rw[k]));
         else if (kind == VP_BALL) f += (r2 < __dmul_rn(w, w)) ? a : 0.0;
         else f += a * exp(-w * sqrt(r2));
         p += 2 + dim;
@@ -287,6 +300,8 @@ struct Loop {
     float ngD_m;                // N_g^D = ngD_m 2^ngD_e
     int ngD_e;
     double nst, ng;
+    double rnst;                // 1 / N_st rounded to nearest
+    bool k_small;               // every axis has at most 2^19 strata (FP64 path, k_plus_u)
     const float2 *tab;
     const double *edges;
 };
@@ -316,6 +331,8 @@ __device__ __forceinline__ Loop make_loop(const Desc *dp, uint32_t t) {
     L.ngD_m = __ldg(&dp->ngD_m);
     L.ngD_e = __ldg(&dp->ngD_e);
     L.nst = (double)L.n_st;
+    L.rnst = __ldg(&dp->strata.rnd[0]);
+    L.k_small = __ldg(&dp->k_small) != 0u;
     L.ng = (double)L.n_g;
     L.tab = (const float2 *)__ldg((const unsigned long long *)&dp->tab);
     L.edges = (const double *)__ldg((const unsigned long long *)&dp->edges);
@@ -527,8 +544,38 @@ __device__ __forceinline__ void point32_p1(const Loop &L, const Strata *S, const
 }
 
 // ---------------------------------------------------------------------------
-// One sample, FP64 path (a1-a3), the oracle's IEEE sequence step by step.
+// One sample, FP64 path (a1-a3): the values of the oracle's IEEE sequence,
+// step by step.  Bound: the FP64 pipe (two lanes of an SM per cycle, 16 cycles
+// per warp instruction), so the steps are formed with as few FP64 instructions
+// as give the same bits: k + u by one subtraction, y by three operations
+// instead of a division, the increment by a round-down addition instead of a
+// floor and two conversions.
 // ---------------------------------------------------------------------------
+// k + u with u = (w + 1/2) 2^-32.  Up to 2^19 strata the sum has at most 52
+// bits, so it is exact: its bits are put below the leading bit of 2^19 (unit
+// in the last place 2^-33) and 2^19 is taken off.  `small`: every axis has at
+// most 2^19 strata; else the sum as written, rounded once.
+__device__ __forceinline__ double k_plus_u(uint32_t k, uint32_t w, bool small) {
+    if (small) {
+        const int lo = (int)((w << 1) | 1u);
+        const int hi = (int)(0x41200000u | (k << 1) | (w >> 31));
+        return __dsub_rn(__hiloint2double(hi, lo), 524288.0);
+    }
+    return __dadd_rn((double)k, u01_f64(w));
+}
+
+// a / n for a whole n in [1, 2^31) and finite a = 0 or a >= 2^-900, with
+// rn = 1/n rounded to nearest: q = a rn is within two units in the last place
+// of the quotient Q, the residual a - n q is exact (a fused multiply-add), and
+// adding it times rn leaves an error below 2^-51 units before the last
+// rounding, while Q is never a midpoint of two doubles (2^53 < its odd part)
+// and at least 1/(2n) units from one: the result is the correctly rounded
+// quotient, as a division gives it (Markstein, IBM J. Res. Dev. 34 (1990)).
+__device__ __forceinline__ double div_by(double a, double n, double rn) {
+    const double q = __dmul_rn(a, rn);
+    return __fma_rn(__fma_rn(-n, q, a), rn, q);
+}
+
 template <int DMAX, int KIND, bool AX>
 __device__ __forceinline__ void point64(const Loop &L, const Strata *S, const double *prm,
                                         uint32_t h, uint32_t j,
@@ -544,13 +591,20 @@ __device__ __forceinline__ void point64(const Loop &L, const Strata *S, const do
             for (int l = 0; l < 4; ++l) {
                 const int mu = 4 * q + l;
                 if (mu < DMAX && mu < L.dim) {
-                    const double u = u01_f64(lane_of(r, l));
-                    const double y =
-                        __ddiv_rn(__dadd_rn((double)kd[mu], u), AX ? S->nd[mu] : L.nst);
+                    const double a = k_plus_u(kd[mu], lane_of(r, l), L.k_small);
+                    // a / N_st, correctly rounded (see div_by)
+                    const double y = AX ? div_by(a, S->nd[mu], S->rnd[mu])
+                                        : div_by(a, L.nst, L.rnst);
                     const double yng = __dmul_rn(y, L.ng);
-                    int i = (int)floor(yng);
-                    i = i > L.n_g - 1 ? L.n_g - 1 : i;
-                    const double delta = __dsub_rn(yng, (double)i);
+                    // floor(yng) for 0 <= yng < 2^31 by a round-down add of 2^52
+                    const double big = __dadd_rd(yng, 4503599627370496.0);
+                    int i = __double2loint(big);
+                    double fl = __dsub_rn(big, 4503599627370496.0);
+                    if (i > L.n_g - 1) {
+                        i = L.n_g - 1;
+                        fl = (double)i;
+                    }
+                    const double delta = __dsub_rn(yng, fl);
                     const double *e = L.edges + (size_t)mu * (size_t)(L.n_g + 1);
                     const double e0 = __ldg(e + i), e1 = __ldg(e + i + 1);
                     const double dx = __dsub_rn(e1, e0);

@@ -74,6 +74,7 @@ struct Strata {
     int32_t shift[kMaxDim];    //   t = umulhi(magic[mu], h); shift 0: n[mu] = 1
     float c32[kMaxDim];        // N_g / n[mu] (FP32 path)
     double nd[kMaxDim];        // n[mu] (FP64 path)
+    double rnd[kMaxDim];       // 1 / n[mu] rounded to nearest (FP64 path)
 };
 
 // Read-only (per iteration) description of one integral.
@@ -86,6 +87,7 @@ struct Desc {
     uint32_t key0, key1;       // Philox key (seed lo, hi)
     uint32_t n_tree;           // ceil(n_hc / kTreeBlock)
     uint32_t uniform;          // 1: the same strata on every axis (the task kernel's case)
+    uint32_t k_small;          // 1: at most 2^19 strata on every axis (FP64 path)
     int64_t n_ev;
     uint64_t n_hc;             // N_h = prod_mu strata[mu] (N_st^D when uniform)
     double omega;              // y-volume of a hypercube, 1 / N_h
@@ -104,7 +106,7 @@ struct Desc {
     // device buffers (all owned by the set)
     double *edges;     // [dim][n_g + 1] FP64 grid
     float2 *tab;       // [dim][n_g] {x_i, dx_i}, FP32 mirror of the grid
-    const double *prm;  // integrand blob as given (FP64 path)
+    const double *prm;  // integrand blob as given, then constants derived from it (FP64 path)
     const float *prm32; // FP32 constants derived from the blob (FP32 path)
     uint32_t *n_h;     // [n_hc]
     uint64_t *off;     // [n_hc + 1] exclusive offsets; off[n_hc] = samples this iteration

@@ -955,7 +955,7 @@ static cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, cudaSt
 //   C[k][l] = sum_h Omega^2 (X2_h[k,l]/n_h - (X1_h[k]/n_h)(X1_h[l]/n_h)) / (n_h - 1)
 // (diagonal terms clamped at zero), every sum in the fixed order of the
 // one-integral sums: blocks of kTreeBlock hypercubes by pairwise halving, then
-// an adjacent pairwise tree over the blocks.  One CTA per block; the last CTA
+// an adjacent pairwise tree over the blocks.  The last CTA
 // to finish combines the blocks and writes the iteration's row of the
 // history.  Launched between the sampling kernel and k_estimate (which
 // advances the iteration counter); it clears the other buffer of X1, X2 for
@@ -964,49 +964,92 @@ static cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, cudaSt
 constexpr int kMultiThreads = 256;
 constexpr int kMultiMaxBlocks = (int)(kMultiMaxHc / kTreeBlock);  // 4096
 
-__device__ __forceinline__ double multi_term(const Desc &d, const double *X1, const double *X2,
-                                             int M, int s, uint64_t h) {
-    if (h >= d.n_hc) return 0.0;
-    const double n = (double)d.n_h[h];
-    const double om = d.omega;
-    if (s < M) return __dmul_rn(om, __ddiv_rn(X1[h * M + s], n));
-    int k = 0, q = s - M;  // (k, l) of triangle entry q
-    while (q >= M - k) {
-        q -= M - k;
-        ++k;
-    }
-    const int l = k + q;
-    const uint64_t T = (uint64_t)M * (M + 1) / 2;
-    const double mk = __ddiv_rn(X1[h * M + k], n), ml = __ddiv_rn(X1[h * M + l], n);
-    double c = __dsub_rn(__ddiv_rn(X2[h * T + (s - M)], n), __dmul_rn(mk, ml));
-    if (k == l && c < 0.0) c = 0.0;
-    return __ddiv_rn(__dmul_rn(__dmul_rn(om, om), c), __dsub_rn(n, 1.0));
+// x / n from rn = 1/n rounded to nearest (whole n < 2^32): the product
+// corrected once by its exact residual, the correctly rounded quotient unless
+// x lies near the underflow limit; overflow and NaN pass unchanged.
+__device__ __forceinline__ double over_n(double x, double n, double rn) {
+    const double q = __dmul_rn(x, rn);
+    const double c = __fma_rn(__fma_rn(-n, q, x), rn, q);
+    return (__double2hiint(q) & 0x7ff00000) == 0x7ff00000 ? q : c;
 }
 
-__global__ void __launch_bounds__(kMultiThreads) k_estimate_multi(const Desc *desc) {
+// n_h and what its terms need of it.
+struct MultiH {
+    double n, rn, n1, rn1;  // n_h, 1/n_h, n_h - 1, 1/(n_h - 1)
+};
+__device__ __forceinline__ MultiH multi_h(const Desc &d, uint64_t h) {
+    MultiH v = {2.0, 0.5, 1.0, 1.0};
+    if (h >= d.n_hc) return v;
+    const uint32_t n = d.n_h[h];
+    v.n = u32_to_f64(n);
+    v.n1 = u32_to_f64(n - 1u);
+    v.rn = n < (uint32_t)kInvTab ? __ldg(d.inv_tab + 4 * (size_t)n) : recip_u32(n);
+    v.rn1 = n - 1u < (uint32_t)kInvTab ? __ldg(d.inv_tab + 4 * (size_t)(n - 1u)) : recip_u32(n - 1u);
+    return v;
+}
+
+// Term of hypercube h in series s: s < M the mean of output s, else the
+// covariance entry (k, l).
+__device__ __forceinline__ double multi_term(const Desc &d, const double *X1, const double *X2,
+                                             int M, int s, int k, int l, uint64_t h,
+                                             const MultiH &v) {
+    if (h >= d.n_hc) return 0.0;
+    const double om = d.omega;
+    if (s < M) return __dmul_rn(om, over_n(X1[h * M + s], v.n, v.rn));
+    const uint64_t T = (uint64_t)M * (M + 1) / 2;
+    const double mk = over_n(X1[h * M + k], v.n, v.rn);
+    const double ml = k == l ? mk : over_n(X1[h * M + l], v.n, v.rn);
+    double c = __dsub_rn(over_n(X2[h * T + (s - M)], v.n, v.rn), __dmul_rn(mk, ml));
+    if (k == l && c < 0.0) c = 0.0;
+    return over_n(__dmul_rn(__dmul_rn(om, om), c), v.n1, v.rn1);
+}
+
+// The adjacent pairwise tree over 32 values, one per lane (the result in lane 0).
+__device__ __forceinline__ double warp_adjacent(double x) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) x = __dadd_rn(x, __shfl_down_sync(0xffffffffu, x, o));
+    return x;
+}
+
+// CTA (block of hypercubes, group of `per` series).  Bound: the FP64 pipe.
+// One CTA per block for all 44 series of 8 outputs left 128 of the 152 SMs
+// idle at 24 blocks (24,389 hypercubes) and divided four times per term.
+__global__ void __launch_bounds__(kMultiThreads) k_estimate_multi(const Desc *desc, int per) {
     __shared__ double sh[kMultiThreads];
-    __shared__ double tree[kMultiMaxBlocks];
     __shared__ bool s_last;
     pdl_wait();
     const Desc &d = *desc;
     const int M = d.n_out, T = M * (M + 1) / 2, NS = M + T;
+    const uint32_t n_grp = (uint32_t)((NS + per - 1) / per), n_blk = gridDim.x / n_grp;
     const uint32_t t_it = __ldcg(&d.st->t);  // the iteration being estimated
     const uint64_t par = t_it & 1u;
     const double *X1 = d.x1 + par * d.n_hc * M, *X2 = d.x2 + par * d.n_hc * T;
-    const uint32_t blk = blockIdx.x, t = threadIdx.x;
+    const uint32_t blk = blockIdx.x / n_grp, grp = blockIdx.x % n_grp, t = threadIdx.x;
     const uint64_t h0 = (uint64_t)blk * kTreeBlock;
-    for (int s = 0; s < NS; ++s) {
+    MultiH v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = multi_h(d, h0 + t + 256u * q);
+    const int s0 = (int)grp * per, s1 = min(s0 + per, NS);
+    for (int s = s0; s < s1; ++s) {
+        int k = 0, l = 0;
+        if (s >= M) {  // (k, l) of triangle entry s - M
+            l = s - M;
+            while (l >= M - k) {
+                l -= M - k;
+                ++k;
+            }
+            l += k;
+        }
         // halving over the block's 1024 terms: i += i + 512, then i += i + 256
         // (thread t holds terms t, t + 256, t + 512, t + 768), then in shared
         // memory down to 32 terms, then by shuffles
-        const double v0 = multi_term(d, X1, X2, M, s, h0 + t);
-        const double v1 = multi_term(d, X1, X2, M, s, h0 + t + 256);
-        const double v2 = multi_term(d, X1, X2, M, s, h0 + t + 512);
-        const double v3 = multi_term(d, X1, X2, M, s, h0 + t + 768);
-        sh[t] = __dadd_rn(__dadd_rn(v0, v2), __dadd_rn(v1, v3));
+        double w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] = multi_term(d, X1, X2, M, s, k, l, h0 + t + 256u * q, v[q]);
+        sh[t] = __dadd_rn(__dadd_rn(w[0], w[2]), __dadd_rn(w[1], w[3]));
         __syncthreads();
-        for (int w = 128; w >= 32; w >>= 1) {
-            if (t < (uint32_t)w) sh[t] = __dadd_rn(sh[t], sh[t + w]);
+        for (int o = 128; o >= 32; o >>= 1) {
+            if (t < (uint32_t)o) sh[t] = __dadd_rn(sh[t], sh[t + o]);
             __syncthreads();
         }
         if (t < 32) {
@@ -1016,12 +1059,13 @@ __global__ void __launch_bounds__(kMultiThreads) k_estimate_multi(const Desc *de
         }
         __syncthreads();
     }
-    {  // the other buffer, zero for the next iteration (this block's hypercubes)
+    {  // the other buffer, zero for the next iteration (this block's hypercubes, shared by its CTAs)
         const uint64_t hb = min((uint64_t)kTreeBlock, d.n_hc - h0);
         double *Y1 = d.x1 + (par ^ 1u) * d.n_hc * M + h0 * M;
         double *Y2 = d.x2 + (par ^ 1u) * d.n_hc * T + h0 * T;
-        for (uint64_t i = t; i < hb * M; i += kMultiThreads) Y1[i] = 0.0;
-        for (uint64_t i = t; i < hb * T; i += kMultiThreads) Y2[i] = 0.0;
+        const uint64_t i0 = grp * kMultiThreads + t, stride = (uint64_t)n_grp * kMultiThreads;
+        for (uint64_t i = i0; i < hb * M; i += stride) Y1[i] = 0.0;
+        for (uint64_t i = i0; i < hb * T; i += stride) Y2[i] = 0.0;
     }
     __threadfence();
     __syncthreads();
@@ -1029,22 +1073,32 @@ __global__ void __launch_bounds__(kMultiThreads) k_estimate_multi(const Desc *de
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    uint32_t P = 1;
-    while (P < gridDim.x) P <<= 1;
-    for (int s = 0; s < NS; ++s) {
-        for (uint32_t i = t; i < P; i += kMultiThreads)
-            tree[i] = i < gridDim.x ? __ldcg(d.mpart + (size_t)i * NS + s) : 0.0;
-        __syncthreads();
-        for (uint32_t w = 1; w < P; w <<= 1) {
-            for (uint32_t i = t * 2 * w; i < P; i += kMultiThreads * 2 * w)
-                tree[i] = __dadd_rn(tree[i], tree[i + w]);
-            __syncthreads();
+    // the adjacent pairwise tree over the blocks (zeros up to a power of two),
+    // one warp per series: 32 consecutive blocks at a time, the sums of those
+    // kept lane by lane for the next level (at most 4 x 32 of them)
+    const int lane = (int)(t & 31u);
+    for (int s = (int)(t >> 5); s < NS; s += kMultiThreads / 32) {
+        double r[kMultiMaxBlocks / 1024];
+#pragma unroll
+        for (int a = 0; a < kMultiMaxBlocks / 1024; ++a) {
+            r[a] = 0.0;
+            if ((uint32_t)a * 1024u < n_blk) {
+                const uint32_t n_c = min((n_blk - a * 1024u + 31u) / 32u, 32u);
+                for (uint32_t c = 0; c < n_c; ++c) {
+                    const uint32_t i = a * 1024u + c * 32u + lane;
+                    double x = i < n_blk ? __ldcg(d.mpart + (size_t)i * NS + s) : 0.0;
+                    x = __shfl_sync(0xffffffffu, warp_adjacent(x), 0);
+                    if ((uint32_t)lane == c) r[a] = x;
+                }
+                r[a] = warp_adjacent(r[a]);
+            }
         }
-        if (t == 0 && t_it < (uint32_t)d.hist_cap) {
-            if (s < M) d.hist_im[(size_t)t_it * M + s] = tree[0];
-            else d.hist_cm[(size_t)t_it * T + (s - M)] = tree[0];
+        static_assert(kMultiMaxBlocks / 1024 == 4, "the last two levels");
+        const double tot = __dadd_rn(__dadd_rn(r[0], r[1]), __dadd_rn(r[2], r[3]));
+        if (lane == 0 && t_it < (uint32_t)d.hist_cap) {
+            if (s < M) d.hist_im[(size_t)t_it * M + s] = tot;
+            else d.hist_cm[(size_t)t_it * T + (s - M)] = tot;
         }
-        __syncthreads();
     }
     if (t == 0) d.st->done_multi = 0u;
 }
@@ -1087,10 +1141,16 @@ cudaError_t launch_partials(const Desc *desc, double *buf, uint64_t n, int dir, 
                       desc, buf, dir);
 }
 
-cudaError_t launch_estimate_multi(const Desc *desc, uint32_t n_blocks, cudaStream_t s) {
+cudaError_t launch_estimate_multi(const Desc *desc, uint32_t n_blocks, int n_out,
+                                  cudaStream_t s) {
     // (programmatic serialisation: waits for the sampling kernel in pdl_wait;
     // it never triggers early, so k_estimate after it sees its whole result)
-    return launch_pdl(k_estimate_multi, dim3(n_blocks), dim3(kMultiThreads), s, desc);
+    // One series per CTA while that is what fills the GPU; four (one 32-byte
+    // sector of a hypercube's products) once blocks alone do.
+    const int per = n_blocks < 64u ? 1 : 4;
+    const int NS = n_out + n_out * (n_out + 1) / 2;
+    const uint32_t n_grp = (uint32_t)((NS + per - 1) / per);
+    return launch_pdl(k_estimate_multi, dim3(n_blocks * n_grp), dim3(kMultiThreads), s, desc, per);
 }
 
 cudaError_t launch_chunks(const Desc *desc, const uint32_t *members, int n_group,

@@ -323,6 +323,17 @@ vp_status vp::validate(const vp_params *p, const vp_integrand *f, Member &mb) {
                 for (int m = 0; m < stride - 1; ++m)
                     mb.prm32.push_back(m < P ? (float)q[6 + np + i * P + m] : 0.0f);
             }
+        // FP64: after the blob, the reciprocals of the divisors of r^2 as
+        // pairs of doubles (see f_post64), or a zero flag
+        const double dn = 2.0 * sy * sy, dw = 200.0 * sy * sy;
+        const double lim = std::ldexp(1.0, 400);
+        const bool fast = dn > 1.0 / lim && dw < lim;
+        mb.prm.push_back(fast ? 1.0 : 0.0);
+        for (double b : {dn, dw}) {
+            const double hi = fast ? 1.0 / b : 0.0;
+            mb.prm.push_back(hi);
+            mb.prm.push_back(fast ? std::fma(-hi, b, 1.0) * hi : 0.0);
+        }
     } else {
         // per peak {a, k, 0, 0, c[D], pad}: a multiple of 4 floats
         const int K = (int)q[0];
@@ -1170,7 +1181,7 @@ static vp_status set_iterate(Set &s, cudaStream_t stream, bool refine_too = fals
     if (cap != cudaStreamCaptureStatusActive) ++s.iters;
     for (int i = 0; i < n; ++i)
         if (s.m[i].n_out > 1)  // several outputs (App. B), before the counter advances
-            CU(launch_estimate_multi(s.d_desc + i, s.m[i].n_tree, stream));
+            CU(launch_estimate_multi(s.d_desc + i, s.m[i].n_tree, s.m[i].n_out, stream));
     if (refine_too && s.any_refine) {  // the step graph: a8 beside a6 and a7
         vp_status st = fork_refine(s, stream);
         if (st != VP_OK) return st;

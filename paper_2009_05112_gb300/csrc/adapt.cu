@@ -178,6 +178,7 @@ __device__ __forceinline__ double damp_tn32(double t, float2 L, const Desc &d) {
 // with no exchange between the CTAs of a block.
 // ---------------------------------------------------------------------------
 constexpr int kEstCtas = 4;
+static_assert(kSmallBlocks * kEstCtas <= 16, "one cluster");
 
 // The state fields the last step reads, loaded early by every CTA's thread 0
 // (they change only in that step, so the loads overlap the sums instead of
@@ -188,7 +189,7 @@ struct EstPre {
 };
 __device__ void finish_estimate(const Desc &d, double I, double V, double Sd, int mode,
                                 const EstPre &pre);
-__device__ __forceinline__ void block_levels(const Desc &d, uint64_t dst, double *red);
+__device__ __forceinline__ void block_levels(double *out, double *red);
 __device__ __forceinline__ void estimate_last_cta(const Desc &d, uint32_t n_cta, int mode,
                                                   const EstPre &pre, double *red, bool *s_last,
                                                   bool residues = false);
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(256, 4)
     // mod 4 (term i and term i + s, s a multiple of 4): on this CTA's terms
     // 4t + q they are the levels 128 .. 1 over t; the last two levels (2, 1)
     // join the four classes' sums, in the last CTA
-    block_levels(d, 3 * (uint64_t)d.n_tree + 12 * (uint64_t)k + 3 * (uint64_t)q, red);
+    block_levels(d.part + 3 * (size_t)d.n_tree + 12 * (size_t)k + 3 * (size_t)q, red);
     estimate_last_cta(d, d.n_tree * kEstCtas, mode, pre, red, &s_last, true);
 }
 
@@ -304,10 +305,10 @@ __global__ void __launch_bounds__(256, 4)
 // (red = 3 x 256 doubles in shared memory) holds value t of series c -- in
 // the wide form the sum of terms t, t + 256, t + 512, t + 768 of a block (its
 // first two halving levels), in the four-CTA form the term 4t + q; the
-// levels 128 .. 1 leave the sum in part[dst + c] (block_levels).  Then, once
+// levels 128 .. 1 leave the sum in out[c] (block_levels).  Then, once
 // per CTA, the ticket and in the last CTA of the integral the block sums in
 // the fixed tree order and the iteration's bookkeeping (estimate_last_cta).
-__device__ __forceinline__ void block_levels(const Desc &d, uint64_t dst, double *red) {
+__device__ __forceinline__ void block_levels(double *out, double *red) {
     const int t = threadIdx.x;
     double *r0 = red, *r1 = red + 256, *r2 = red + 512;
     __syncthreads();
@@ -326,7 +327,7 @@ __device__ __forceinline__ void block_levels(const Desc &d, uint64_t dst, double
         const double *r = w == 0 ? r0 : (w == 1 ? r1 : r2);
         double x = __dadd_rn(r[l], r[l + 32]);
         for (int s = 16; s >= 1; s >>= 1) x = __dadd_rn(x, __shfl_down_sync(0xffffffffu, x, s));
-        if (l == 0) d.part[dst + w] = x;
+        if (l == 0) out[w] = x;
     }
 }
 
@@ -413,11 +414,23 @@ __global__ void __launch_bounds__(256, 4)
         red[t] = __dadd_rn(__dadd_rn(v0.a, v2.a), __dadd_rn(v1.a, v3.a));
         red[256 + t] = __dadd_rn(__dadd_rn(v0.b, v2.b), __dadd_rn(v1.b, v3.b));
         red[512 + t] = __dadd_rn(__dadd_rn(v0.c, v2.c), __dadd_rn(v1.c, v3.c));
-        block_levels(d, 3 * (uint64_t)k, red);
+        block_levels(d.part + 3 * (size_t)k, red);
     }
     estimate_last_cta(d, (d.n_tree + (uint32_t)group - 1u) / (uint32_t)group, mode, pre, red,
                       &s_last);
 }
+
+// N_ev / sum d of the allocation (0: not a normal number, the exact quotient
+// is taken throughout).
+__device__ __forceinline__ double alloc_c_of(const Desc &d, double Sd, double inv_sum_d) {
+    const double c = d.n_ev_d * inv_sum_d;
+    const bool normal = Sd >= 2.2250738585072014e-308 && c >= 2.2250738585072014e-308 &&
+                        c <= 1.7976931348623157e308;
+    return normal ? c : 0.0;
+}
+// d_h >= 2^-1021 keeps N_ev d_h normal for every N_ev >= 1 (a constant: no
+// FP64 division in the serial step; the rare d_h below it take the exact quotient)
+constexpr double kAllocDmin = 4.4501477170144028e-308;
 
 // The iteration's totals I_j, sigma_j^2 and sum d recorded in the state (one
 // thread): history, the FP32 path's scale, the iteration count and, for a
@@ -429,16 +442,8 @@ __device__ void finish_estimate(const Desc &d, double I, double V, double Sd, in
     V *= d.omega2;
     st->sum_d = Sd;
     st->inv_sum_d = Sd > 0.0 ? 1.0 / Sd : 0.0;
-    {
-        const double c = d.n_ev_d * st->inv_sum_d;
-        const bool normal = Sd >= 2.2250738585072014e-308 && c >= 2.2250738585072014e-308 &&
-                            c <= 1.7976931348623157e308;
-        st->alloc_c = normal ? c : 0.0;
-        // d_h >= 2^-1021 keeps N_ev d_h normal for every N_ev >= 1 (a constant:
-        // no FP64 division in this serial step; the rare d_h below it take the
-        // exact quotient)
-        st->alloc_dmin = 4.4501477170144028e-308;
-    }
+    st->alloc_c = alloc_c_of(d, Sd, st->inv_sum_d);
+    st->alloc_dmin = kAllocDmin;
     if (mode == 0) {
         const uint32_t tt = pre.t;
         if (tt < (uint32_t)d.hist_cap) {
@@ -750,6 +755,101 @@ __global__ void __launch_bounds__(kSubH, 4) k_offsets_wide(const Desc *desc,
                 if (h0 + q < d.n_hc) d.off[h0 + q] = base + e[q];
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// k_adapt_small: k_estimate, k_alloc and k_offsets of one integral of at most
+// 4096 hypercubes (kSmallBlocks blocks) in one launch, on one cluster.  These
+// sizes are latency-bound: the three launches spend their time in launches,
+// tickets and last-CTA passes over L2, which the cluster replaces by three
+// barriers and loads from its CTAs' shared memory.  CTA 4k + q first takes the
+// terms 4t + q of block k, as k_estimate does (the same sums in the same
+// order), every CTA adds the block sums itself, allocates n_h of its
+// hypercubes from the d_h it still holds, then takes the quarter q of block k
+// in order for the offsets.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_adapt_small(const Desc *desc) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ double red[3 * 256];
+    __shared__ double s_part[3], s_sum[3];
+    __shared__ uint32_t s_n[256], s_w[8], s_tot;
+    pdl_wait();
+    pdl_trigger();
+    const Desc &d = desc[0];
+    const int rank = (int)cl.block_rank(), cs = (int)cl.num_blocks();
+    const int q = rank & (kEstCtas - 1), k = rank / kEstCtas, t = threadIdx.x;
+    const uint32_t par = d.st->t & 1u;
+    EstPre pre = {0u, 0u, 0ull, 0ull};
+    if (t == 0 && rank == 0) {
+        pre.t = d.st->t;
+        pre.status = d.st->status;
+        pre.n_samples = d.st->n_samples;
+        pre.n_eval_total = d.st->n_eval_total;
+    }
+    const D3 v = hcube_terms(d, (uint64_t)k * kTreeBlock + 4 * t + q, 0, par);
+    {  // clear the other histogram buffer
+        const int bins = d.dim * d.n_g;
+        double *hs = d.hsum + (size_t)(par ^ 1u) * bins;
+        uint32_t *hc = d.hcnt + (size_t)(par ^ 1u) * bins;
+        for (int i = rank * 256 + t; i < bins; i += cs * 256) {
+            hs[i] = 0.0;
+            hc[i] = 0u;
+        }
+    }
+    red[t] = v.a;
+    red[256 + t] = v.b;
+    red[512 + t] = v.c;
+    block_levels(s_part, red);
+    cl.sync();  // (every CTA has read the state; the class sums are there)
+    const int w = t >> 5, lane = t & 31;
+    if (w < 3) {  // series w: lane l takes block l, then the adjacent pairwise tree
+        double x = 0.0;
+        if (lane < (int)d.n_tree) {
+            const double c0 = cl.map_shared_rank(s_part, 4 * lane)[w];
+            const double c1 = cl.map_shared_rank(s_part, 4 * lane + 1)[w];
+            const double c2 = cl.map_shared_rank(s_part, 4 * lane + 2)[w];
+            const double c3 = cl.map_shared_rank(s_part, 4 * lane + 3)[w];
+            x = __dadd_rn(__dadd_rn(c0, c2), __dadd_rn(c1, c3));
+        }
+#pragma unroll
+        for (int o = 1; o < kSmallBlocks; o <<= 1)
+            if ((uint32_t)o < d.n_tree) x = __dadd_rn(x, __shfl_down_sync(0xffffffffu, x, o));
+        if (lane == 0) s_sum[w] = x;
+    }
+    __syncthreads();
+    if (rank == 0 && t == 0) finish_estimate(d, s_sum[0], s_sum[1], s_sum[2], 0, pre);
+    AllocK K;
+    K.n_ev_d = d.n_ev_d;
+    K.sum_d = s_sum[2];
+    K.c = alloc_c_of(d, K.sum_d, K.sum_d > 0.0 ? 1.0 / K.sum_d : 0.0);
+    K.dmin = kAllocDmin;
+    K.n_hc = d.n_hc;
+    K.plus2 = d.plus2 != 0;
+    const bool ok = finite_bits(K.sum_d);  // (the same in every CTA)
+    s_n[t] = ok && (uint64_t)k * kTreeBlock + 4 * t + q < d.n_hc ? alloc_one(v.c, K, 0) : 0u;
+    cl.sync();
+    if (!ok) {  // the allocation is kept (every remote read was before the barrier)
+        if (rank == 0 && t == 0) d.st->status |= kStatusNonFinite;
+        return;
+    }
+    const int j = q * 256 + t;  // hypercube j of block k is term j / 4 of class j mod 4
+    const uint32_t n = cl.map_shared_rank(s_n, 4 * k + (j & 3))[j >> 2];
+    const uint64_t h = (uint64_t)k * kTreeBlock + j;
+    if (h < d.n_hc) d.n_h[h] = n;
+    uint32_t tot;
+    const uint32_t ex = cta_exclusive_scan32(n, s_w, &tot);
+    if (t == 0) s_tot = tot;
+    cl.sync();
+    uint32_t base = lane < rank ? *cl.map_shared_rank(&s_tot, lane) : 0u;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) base += __shfl_xor_sync(0xffffffffu, base, o);
+    if (h < d.n_hc) d.off[h] = (uint64_t)(base + ex);
+    if (rank == cs - 1 && t == 0) {
+        d.off[d.n_hc] = (uint64_t)(base + tot);
+        d.st->n_samples = (uint64_t)(base + tot);
+    }
+    cl.sync();  // keep this CTA's shared memory alive until every remote read is done
 }
 
 // ---------------------------------------------------------------------------
@@ -1183,6 +1283,51 @@ cudaError_t launch_estimate(const Desc *desc, const uint32_t *tree_base, int n_i
     }
     return launch_pdl(k_estimate, dim3(n_blocks * kEstCtas), dim3(256), s, desc, tree_base, n_int,
                       mode);
+}
+
+// The cluster launch of k_adapt_small: 4, 8 or 16 CTAs (CTAs beyond the blocks
+// hold no hypercubes).
+static void small_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&at)[2],
+                         uint32_t n_blocks, cudaStream_t s) {
+    const unsigned cs = n_blocks <= 1 ? 4u : (n_blocks <= 2 ? 8u : 16u);
+    cfg = {};
+    cfg.gridDim = dim3(cs);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cs;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+}
+
+bool adapt_small_fits(uint32_t n_blocks) {
+    if (n_blocks > (uint32_t)kSmallBlocks) return false;
+    if (cudaFuncSetAttribute(k_adapt_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[2];
+    small_config(cfg, at, n_blocks, nullptr);
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_adapt_small, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n >= 1;
+}
+
+cudaError_t launch_adapt_small(const Desc *desc, uint32_t n_blocks, cudaStream_t s) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[2];
+    small_config(cfg, at, n_blocks, s);
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, k_adapt_small, desc);
 }
 
 cudaError_t launch_alloc(const Desc *desc, const uint32_t *tree_base, int n_int,

@@ -104,6 +104,7 @@ struct Set {
     uint32_t n_tree_total = 0, n_axis_total = 0;
     int max_ng = 1;
     bool any_refine = false;
+    bool adapt_small = false;  // the step graph takes k_adapt_small (one integral, few hypercubes)
     cudaStream_t last = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     // the refinement (a8) runs on a side stream beside the estimate and the
@@ -758,6 +759,7 @@ static vp_status set_create(Set &s, int n, const vp_params *ps, const vp_integra
     CU(cudaStreamSynchronize(stream));
     s.n_tree_total = tree_base[n];
     s.n_axis_total = axis_base[n];
+    s.adapt_small = n == 1 && adapt_small_fits(s.n_tree_total);
     for (auto &g : s.groups) {
         if (!g.one) continue;
         const Desc &d = s.h_desc[g.members[0]];
@@ -1186,7 +1188,10 @@ static vp_status set_iterate(Set &s, cudaStream_t stream, bool refine_too = fals
         vp_status st = fork_refine(s, stream);
         if (st != VP_OK) return st;
     }
-    CU(launch_estimate(s.d_desc, s.d_tree_base, n, s.n_tree_total, 0, stream, set_prec(s)));
+    if (refine_too && s.adapt_small)  // the step graph: a6 and a7 in one launch
+        CU(launch_adapt_small(s.d_desc, s.n_tree_total, stream));
+    else
+        CU(launch_estimate(s.d_desc, s.d_tree_base, n, s.n_tree_total, 0, stream, set_prec(s)));
     s.last = stream;
     return VP_OK;
 }
@@ -1198,7 +1203,8 @@ static vp_status set_adapt(Set &s, cudaStream_t stream, bool refine_forked = fal
         vp_status st = fork_refine(s, stream);
         if (st != VP_OK) return st;
     }
-    CU(launch_alloc(s.d_desc, s.d_tree_base, n, s.n_tree_total, stream, 0));
+    if (!(refine_forked && s.adapt_small))
+        CU(launch_alloc(s.d_desc, s.d_tree_base, n, s.n_tree_total, stream, 0));
     if (s.any_refine) {
         vp_status st = join_refine(s, stream);
         if (st != VP_OK) return st;

@@ -31,6 +31,9 @@ cudaError_t launch_chunks(const Desc *, const uint32_t *, int, uint64_t *, uint3
 cudaError_t launch_estimate(const Desc *, const uint32_t *, int, uint32_t, int, cudaStream_t,
                             int prec = -1);
 cudaError_t launch_estimate_multi(const Desc *, uint32_t, int, cudaStream_t);
+// k_adapt_small (the step graph of one small integral): whether it can run, and its launch.
+bool adapt_small_fits(uint32_t n_blocks);
+cudaError_t launch_adapt_small(const Desc *, uint32_t n_blocks, cudaStream_t);
 cudaError_t launch_alloc(const Desc *, const uint32_t *, int, uint32_t, cudaStream_t, int initial);
 cudaError_t launch_refine(const Desc *, const uint32_t *, int, uint32_t, int, cudaStream_t);
 cudaError_t launch_partials(const Desc *, double *, uint64_t, int dir, cudaStream_t);

@@ -17,6 +17,8 @@ namespace vp {
 constexpr int kMaxDim = 24;        // D limit (largest bucket of the sampling kernel)
 constexpr int kMaxNg = 4096;       // N_g limit (refinement keeps a whole axis in shared memory)
 constexpr int kTreeBlock = 1024;   // hypercubes per block of the fixed-order sum
+// blocks one integral may have for its estimate and allocation to run as one cluster
+constexpr int kSmallBlocks = 4;
 constexpr int kSub = 4;            // CTAs of the allocation kernels per block of kTreeBlock
 constexpr int kSubH = kTreeBlock / kSub;
 constexpr int kMaxPeaks = 64;

@@ -861,11 +861,16 @@ __global__ void __launch_bounds__(256) k_adapt_small(const Desc *desc) {
 //   1. d_i for the owned range plus one halo increment each side; partial sum
 //   2. sum_i d_i = the 8 partials in rank order (identical in every CTA)
 //   3. smoothing, normalisation, compression; local inclusive scan
-//   4. cumulative base of every CTA = the totals of lower ranks
+//   4. cumulative base of every CTA = the totals of lower ranks, added to its
+//      scan
 //   5. new edge k (for k in the owned range) where the cumulative reaches
 //      k sum(c)/N_g: the owning rank is found from the totals, then a binary
-//      search in that rank's local scan, read remotely
+//      search in that rank's cumulative, read remotely
 //   6. edges and the FP32 table {x_i, dx_i} written back.
+// One axis is latency-bound (~14 us); many (a batch, a server's requests) are
+// bound by the FP64 pipe, 16 cycles per warp instruction, so what every thread
+// needs of the cluster (1 / sum, the bases, the step) is formed by one warp,
+// and the searches compare the bits of their nonnegative numbers.
 // ---------------------------------------------------------------------------
 constexpr int kRefineCtas = 8;
 constexpr int kRefineThreads = 128;
@@ -878,6 +883,8 @@ struct RefineShared {
     double C[kRefineSlice];       // local inclusive scan of c
     double xn[kRefineSlice + 1];  // new edges of the owned range (and one more)
     double red[kRefineThreads / 32];
+    double base[kRefineCtas];     // cumulative before each rank's increments
+    double sum, inv_sum, step;    // axis total of raw d, its reciprocal, sum(c)/N_g
     double part;                  // sum of own raw d
     double tot;                   // sum of own c
     int n_own;
@@ -932,13 +939,23 @@ __global__ void __cluster_dims__(kRefineCtas, 1, 1) __launch_bounds__(kRefineThr
     }
     cl.sync();
     // 2. the axis total, in rank order
-    double sum_d = 0.0;
-    for (int q = 0; q < kRefineCtas; ++q) sum_d += *cl.map_shared_rank(&sm.part, q);
-    if (!(sum_d > 0.0) || !isfinite(sum_d)) {  // nothing to refine (reading); uniform
+    const int lane = t & 31, w = t >> 5;
+    if (w == 0) {
+        const double p = lane < kRefineCtas ? *cl.map_shared_rank(&sm.part, lane) : 0.0;
+        double sum = 0.0;
+#pragma unroll
+        for (int q = 0; q < kRefineCtas; ++q) sum += __shfl_sync(0xffffffffu, p, q);
+        if (lane == 0) {
+            sm.sum = sum;
+            sm.inv_sum = 1.0 / sum;
+        }
+    }
+    __syncthreads();
+    if (!(sm.sum > 0.0) || !isfinite(sm.sum)) {  // nothing to refine (reading); uniform
         cl.sync();
         return;
     }
-    const double inv_sum = 1.0 / sum_d;
+    const double inv_sum = sm.inv_sum;
     // 3. smoothing, normalisation, compression; contiguous quarter-slices per thread
     const int n_own = i1 - i0;
     const int per = (n_own + nt - 1) / nt;
@@ -954,9 +971,9 @@ __global__ void __cluster_dims__(kRefineCtas, 1, 1) __launch_bounds__(kRefineThr
         s = s * inv_sum;
         // reading: an unsampled increment keeps the weight of the smallest
         // normal double (the alpha -> 0 limit stays "no refinement")
-        if (s <= 0.0) s = 2.2250738585072014e-308;
+        if (__double_as_longlong(s) <= 0ll) s = 2.2250738585072014e-308;
         double cv;
-        if (s == 1.0) cv = 1.0;
+        if (__double_as_longlong(s) == 0x3ff0000000000000ll) cv = 1.0;
         else {
             const double r = (1.0 - s) / -log(s);
             cv = d.alpha == 1.0 ? r : (d.alpha == 0.5 ? sqrt(r) : pow(r, d.alpha));
@@ -967,7 +984,6 @@ __global__ void __cluster_dims__(kRefineCtas, 1, 1) __launch_bounds__(kRefineThr
     }
     // exclusive prefix of the thread totals (warp shuffles, then warps)
     double inc = local;
-    const int lane = t & 31, w = t >> 5;
     for (int o = 1; o < 32; o <<= 1) {
         const double v = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += v;
@@ -983,29 +999,39 @@ __global__ void __cluster_dims__(kRefineCtas, 1, 1) __launch_bounds__(kRefineThr
     if (t == 0) sm.tot = n_own > 0 ? sm.C[n_own - 1] : 0.0;
     cl.sync();
     // 4. bases of every rank and the axis total of c
-    double base[kRefineCtas];
-    double total = 0.0;
-    for (int q = 0; q < kRefineCtas; ++q) {
-        base[q] = total;
-        total += *cl.map_shared_rank(&sm.tot, q);
+    if (w == 0) {
+        const double p = lane < kRefineCtas ? *cl.map_shared_rank(&sm.tot, lane) : 0.0;
+        double total = 0.0, base = 0.0;
+#pragma unroll
+        for (int q = 0; q < kRefineCtas; ++q) {
+            if (lane == q) base = total;
+            total += __shfl_sync(0xffffffffu, p, q);
+        }
+        if (lane < kRefineCtas) sm.base[lane] = base;
+        if (lane == 0) sm.step = total / (double)n_g;
     }
-    const double delta_d = total / (double)n_g;
-    // 5. new edges k in [max(i0, 1), min(i1, n_g - 1)]
+    __syncthreads();
+    for (int a = t; a < n_own; a += nt) sm.C[a] = sm.base[rank] + sm.C[a];
+    cl.sync();
+    const double delta_d = sm.step;
+    // 5. new edges k in [max(i0, 1), min(i1, n_g - 1)] (every number compared
+    // here is finite and >= 0, so its bits order it)
     for (int k = max(i0, 1) + t; k < min(i1, n_g); k += nt) {
         const double target = (double)k * delta_d;
+        const long long tb = __double_as_longlong(target);
         int q = 0;
-        while (q < kRefineCtas - 1 && base[q + 1] < target) ++q;
-        // rank q holds the crossing: smallest m with base[q] + C_q[m] >= target
+        while (q < kRefineCtas - 1 && __double_as_longlong(sm.base[q + 1]) < tb) ++q;
+        // rank q holds the crossing: smallest m with C_q[m] >= target
         const RefineShared *rs = cl.map_shared_rank(&sm, q);
         const int nq = rs->n_own;
-        int lo = -1, hi = nq - 1;  // base + C[hi] >= target (the last one is, up to rounding)
+        int lo = -1, hi = nq - 1;  // C[hi] >= target (the last one is, up to rounding)
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
-            if (base[q] + rs->C[mid] < target) lo = mid;
+            if (__double_as_longlong(rs->C[mid]) < tb) lo = mid;
             else hi = mid;
         }
         // cumulative at the right end of increment j - 1 = q S + hi
-        const double Cj = base[q] + rs->C[hi];
+        const double Cj = rs->C[hi];
         const double cj = rs->c[hi];
         const double xr = rs->x[hi + 1], xl = rs->x[hi];
         sm.xn[k - i0] = cj > 0.0 ? xr - ((Cj - target) / cj) * (xr - xl) : xr;

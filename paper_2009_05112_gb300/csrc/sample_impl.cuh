@@ -1391,9 +1391,21 @@ __global__ void __launch_bounds__(one_max_threads(DMAX, F64, P1), 1)
         double *X1 = MO ? a.x1 + par * a.n_hc * (uint64_t)a.n_out : nullptr;
         double *X2 = MO ? a.x2 + par * a.n_hc * (uint64_t)(a.n_out * (a.n_out + 1) / 2) : nullptr;
         // (sample indices are 32-bit: an iteration has fewer than 2^32 samples)
-        const uint32_t per_w = n_st / W, extra = n_st - per_w * W;
-        const uint32_t wb = lo + w * per_w + min(w, extra);
-        const uint32_t we = wb + per_w + (w < extra ? 1u : 0u);
+        // few samples per warp: the fewest warps that take no more samples per
+        // lane, each of whole 32s but for a few, spread over the CTAs before
+        // they share one -- 1e4 samples over 2432 warps were 4 lanes of each
+        // warp at work, and the FP64 path, whose warp instructions cost the
+        // same whatever their lanes do, paid for all 32.  (From 9 samples per
+        // lane on the idle lanes cost less than a warp in nine.)
+        uint32_t Ws = W, ws = w;
+        const uint32_t rounds = n_st / (32u * W) + (n_st % (32u * W) != 0u ? 1u : 0u);
+        if (rounds <= 8u && rounds > 0u) {
+            Ws = (n_st + 32u * rounds - 1u) / (32u * rounds);
+            ws = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+        }
+        const uint32_t per_w = n_st / Ws, extra = n_st - per_w * Ws;
+        const uint32_t wb = lo + min(ws, Ws) * per_w + min(ws, extra);
+        const uint32_t we = ws < Ws ? wb + per_w + (ws < extra ? 1u : 0u) : wb;
         // the dynamic tail: chunks of 32 r samples, each warp pulling the next
         // one from the queue as it finishes
         const uint32_t C = 32u * (uint32_t)a.r;

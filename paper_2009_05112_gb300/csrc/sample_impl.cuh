@@ -93,8 +93,10 @@ __device__ __forceinline__ double f_peaks64(int kind, const double *p, int K, in
 #pragma unroll
         for (int mu = 0; mu < DMAX; ++mu) {
             if (mu < dim) {
+                // (one rounding fewer per axis and two FP64 instructions instead
+                // of three; the ball's edge keeps the unfused sum it is compared by)
                 double dx = __dsub_rn(x[mu], c[mu]);
-                r2 = __dadd_rn(r2, __dmul_rn(dx, dx));
+                r2 = kind == VP_BALL ? __dadd_rn(r2, __dmul_rn(dx, dx)) : __fma_rn(dx, dx, r2);
             }
         }
         if (kind == VP_GAUSS) f += a * exp(ratio64(-r2, __dmul_rn(w, w), rw[k]));

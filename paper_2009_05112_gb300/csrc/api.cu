@@ -487,11 +487,11 @@ static vp_status plan_groups(Set &s) {
                         ? sample_occupancy_f64(g.bucket, g.exact, g.kind, true, g.threads, g.smem_one, g.mo)
                         : sample_occupancy_f32(g.bucket, g.exact, g.kind, true, g.threads, g.smem_one, false, g.p1);
         if (g.occ_one < 1) return fail(VP_ECUDA, "sampling kernel cannot be resident (smem %zu)", g.smem_one);
-        // until the autotuner has measured: two CTAs per SM, or one where that
-        // already holds the samples at one per lane (each CTA clears and flushes
-        // histograms of its own)
+        // until the autotuner has measured: two CTAs per SM, or one on the FP64
+        // path where that holds the samples at one per lane (each CTA clears and
+        // flushes histograms of its own)
         const double samples = (double)s.m[g.members[0]].p.n_ev + 2.0 * (double)s.m[g.members[0]].n_hc;
-        g.blocks = s.n_sm * std::min(g.occ_one, samples <= (double)s.n_sm * g.threads ? 1 : 2);
+        g.blocks = s.n_sm * std::min(g.occ_one, g.prec == VP_FP64 && samples <= (double)s.n_sm * g.threads ? 1 : 2);
         if (g.hist_one) {
             // the largest cluster that keeps (nearly) every CTA slot busy
             int best = g.blocks;

@@ -1397,13 +1397,17 @@ __global__ void __launch_bounds__(one_max_threads(DMAX, F64, P1), 1)
         // lane, each of whole 32s but for a few, spread over the CTAs before
         // they share one -- 1e4 samples over 2432 warps were 4 lanes of each
         // warp at work, and the FP64 path, whose warp instructions cost the
-        // same whatever their lanes do, paid for all 32.  (From 9 samples per
-        // lane on the idle lanes cost less than a warp in nine.)
+        // same whatever their lanes do, paid for all 32.  (FP64 up to 8 samples
+        // per lane: beyond it the idle lanes cost less than a warp in nine.
+        // FP32 at one per lane, up to D = 8 and not in parts: its sums depend on
+        // which samples a lane, a warp's combine and a CTA's histogram add.)
         uint32_t Ws = W, ws = w;
-        const uint32_t rounds = n_st / (32u * W) + (n_st % (32u * W) != 0u ? 1u : 0u);
-        if (rounds <= 8u && rounds > 0u) {
-            Ws = (n_st + 32u * rounds - 1u) / (32u * rounds);
-            ws = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+        if constexpr (F64 || DMAX <= 8) {
+            const uint32_t rounds = n_st / (32u * W) + (n_st % (32u * W) != 0u ? 1u : 0u);
+            if (rounds > 0u && rounds <= (F64 ? 8u : 1u) && (F64 || a.n_parts == 0)) {
+                Ws = (n_st + 32u * rounds - 1u) / (32u * rounds);
+                ws = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+            }
         }
         const uint32_t per_w = n_st / Ws, extra = n_st - per_w * Ws;
         const uint32_t wb = lo + min(ws, Ws) * per_w + min(ws, extra);

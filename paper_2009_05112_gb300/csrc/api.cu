@@ -517,7 +517,11 @@ static vp_status plan_groups(Set &s) {
 
 // Task-kernel launch shape of a group: shared-memory histograms when the
 // largest member's fit (with the FP32 constants) in 112 KB, two CTAs per SM at
-// most, tasks of ~1/8 of a CTA's share in whole warp chunks.
+// most, tasks of ~1/8 of a CTA's share in whole warp chunks.  Groups of
+// several FP32 peak integrals up to D = 12 take one CTA of 768 threads per SM
+// where the histograms fit in 220 KB (see k_sample_many); larger dimensions
+// and posteriors keep 256 (posteriors spill at 80 registers: 256 requests 62.7
+// ms against 50.1).
 vp_status vp::group_config_many(const std::vector<const Member *> &m, Group &g, int n_sm) {
     double expect = 0.0;
     int max_bins = 0, max_words = 0;
@@ -539,7 +543,10 @@ vp_status vp::group_config_many(const std::vector<const Member *> &m, Group &g, 
     g.hist_words = max_bins;
     g.prm_words = g.prec == VP_FP64 ? 0 : ((max_words + 3) & ~3);
     const size_t prm_bytes = (size_t)g.prm_words * 4;
-    g.hist_shared = (hist_bytes + prm_bytes <= 112 * 1024) ? 1 : 0;
+    // (one member: the autotuner's task scheme, whose CTAs have 256 threads)
+    const int wide = many_max_threads(bucket_dim(g.bucket), g.prec == VP_FP64, g.kind);
+    if (g.members.size() > 1 && hist_bytes + prm_bytes <= kOneSmemMax) g.threads = wide;
+    g.hist_shared = g.threads > 256 || hist_bytes + prm_bytes <= 112 * 1024 ? 1 : 0;
     g.smem = prm_bytes + (g.hist_shared ? hist_bytes : 0);
     g.one = false;
     g.cs = 1;

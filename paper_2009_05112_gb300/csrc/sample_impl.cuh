@@ -23,6 +23,7 @@
 #pragma once
 
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "vp_internal.cuh"
 
@@ -349,14 +350,14 @@ __device__ __forceinline__ float scale2(float x, int n) {
     return x * __int_as_float((n1 + 127) << 23) * __int_as_float((n2 + 127) << 23);
 }
 
-// Per-integral constants of the sampling loop, read once into registers.
-struct Loop {
+// Per-integral constants of the sampling loop, read once into registers; the
+// Philox round keys apart (Loop: with the rest; LoopS: in shared memory).
+struct LoopBase {
     int dim, n_g, K;
     uint32_t nst_magic;
     int nst_shift;
     uint32_t n_st, calls, iid, t;
     int dw;                     // the grid's d_i from samples weighted by 1/n_h
-    uint32_t rk0[10], rk1[10];  // Philox round keys
     float c32;                  // N_g / N_st
     float ngm1;                 // N_g - 1
     float ngD_m;                // N_g^D = ngD_m 2^ngD_e
@@ -367,9 +368,18 @@ struct Loop {
     const float2 *tab;
     const double *edges;
 };
+struct Loop : LoopBase {
+    uint32_t rk0[10], rk1[10];  // Philox round keys
+};
+// Round keys two rounds to an entry, {k0, k1, k0', k1'}: five 16-byte broadcast
+// loads per Philox call instead of 20 registers held across the sample loop
+// (the task kernel: the one-integral kernel has them in the constant bank).
+struct LoopS : LoopBase {
+    const uint4 *keys;  // [5], shared memory
+};
 
-__device__ __forceinline__ Loop make_loop(const Desc *dp, uint32_t t) {
-    Loop L;
+__device__ __forceinline__ LoopBase make_base(const Desc *dp, uint32_t t) {
+    LoopBase L;
     L.dim = __ldg(&dp->dim);
     L.n_g = __ldg(&dp->n_g);
     L.K = __ldg(&dp->n_peaks);
@@ -380,14 +390,6 @@ __device__ __forceinline__ Loop make_loop(const Desc *dp, uint32_t t) {
     L.iid = __ldg(&dp->integral_id);
     L.dw = __ldg(&dp->d_weighted);
     L.t = t;
-    uint32_t k0 = __ldg(&dp->key0), k1 = __ldg(&dp->key1);
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        L.rk0[r] = k0;
-        L.rk1[r] = k1;
-        k0 += 0x9E3779B9u;
-        k1 += 0xBB67AE85u;
-    }
     L.c32 = __ldg(&dp->ng_over_nst);
     L.ngm1 = (float)(L.n_g - 1);
     L.ngD_m = __ldg(&dp->ngD_m);
@@ -398,6 +400,19 @@ __device__ __forceinline__ Loop make_loop(const Desc *dp, uint32_t t) {
     L.ng = (double)L.n_g;
     L.tab = (const float2 *)__ldg((const unsigned long long *)&dp->tab);
     L.edges = (const double *)__ldg((const unsigned long long *)&dp->edges);
+    return L;
+}
+__device__ __forceinline__ Loop make_loop(const Desc *dp, uint32_t t) {
+    Loop L;
+    *(LoopBase *)&L = make_base(dp, t);
+    uint32_t k0 = __ldg(&dp->key0), k1 = __ldg(&dp->key1);
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        L.rk0[r] = k0;
+        L.rk1[r] = k1;
+        k0 += 0x9E3779B9u;
+        k1 += 0xBB67AE85u;
+    }
     return L;
 }
 
@@ -452,18 +467,22 @@ __device__ __forceinline__ void red_add(uint32_t *p, uint32_t v) {
 }
 
 // Philox4x32-10 with precomputed round keys (same function as philox4x32_10).
-__device__ __forceinline__ U4 philox_rk(U4 c, const uint32_t (&k0)[10], const uint32_t (&k1)[10]) {
+__device__ __forceinline__ U4 philox_round(const U4 &c, uint32_t k0, uint32_t k1) {
+    const uint32_t m0 = 0xD2511F53u, m1 = 0xCD9E8D57u;
+    const uint32_t hi0 = __umulhi(m0, c.a), lo0 = m0 * c.a;
+    const uint32_t hi1 = __umulhi(m1, c.c), lo1 = m1 * c.c;
+    return {hi1 ^ c.b ^ k0, lo1, hi0 ^ c.d ^ k1, lo0};
+}
+__device__ __forceinline__ U4 philox_rk(U4 c, const Loop &L) {
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t m0 = 0xD2511F53u, m1 = 0xCD9E8D57u;
-        const uint32_t hi0 = __umulhi(m0, c.a), lo0 = m0 * c.a;
-        const uint32_t hi1 = __umulhi(m1, c.c), lo1 = m1 * c.c;
-        U4 n;
-        n.a = hi1 ^ c.b ^ k0[r];
-        n.b = lo1;
-        n.c = hi0 ^ c.d ^ k1[r];
-        n.d = lo0;
-        c = n;
+    for (int r = 0; r < 10; ++r) c = philox_round(c, L.rk0[r], L.rk1[r]);
+    return c;
+}
+__device__ __forceinline__ U4 philox_rk(U4 c, const LoopS &L) {
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+        const uint4 k = L.keys[r];
+        c = philox_round(philox_round(c, k.x, k.y), k.z, k.w);
     }
     return c;
 }
@@ -471,28 +490,44 @@ __device__ __forceinline__ U4 philox_rk(U4 c, const uint32_t (&k0)[10], const ui
 // The strata constants of axis mu: per axis (AX, from S) or the one count
 // every axis shares (from L).
 template <bool AX>
-__device__ __forceinline__ float c32_of(const Loop &L, const Strata *S, int mu) {
+__device__ __forceinline__ float c32_of(const LoopBase &L, const Strata *S, int mu) {
     return AX ? S->c32[mu] : L.c32;
 }
 
 // FP32 per-hypercube offsets kc[mu] = (k_mu - 1 + 2^-24) N_g/s_mu so that
 // y N_g = (1 + m 2^-23) N_g/s_mu + kc with m = r >> 9, i.e. u = (m + 1/2) 2^-23.
 template <int DMAX, bool AX>
-__device__ __forceinline__ void hcube_offsets(const Loop &L, const Strata *S,
+__device__ __forceinline__ void hcube_offsets(const LoopBase &L, const Strata *S,
                                               const uint32_t (&kd)[DMAX], float (&kc)[DMAX]) {
 #pragma unroll
     for (int mu = 0; mu < DMAX; ++mu)
         kc[mu] = ((float)kd[mu] - 0.99999994039535522461f) * c32_of<AX>(L, S, mu);
 }
 
+// Increment indices (below kMaxNg = 4096) of a sample, FP32 path: above D = 12
+// two to a register, which is what keeps the sample loop's arrays of 24 axes
+// out of local memory.
+template <int DMAX> struct Idx {
+    static constexpr bool kPack = DMAX > 12;
+    uint32_t v[kPack ? (DMAX + 1) / 2 : DMAX];
+    __device__ __forceinline__ void set(int mu, int i) {
+        if (!kPack) v[mu] = (uint32_t)i;
+        else if (mu & 1) v[mu >> 1] |= (uint32_t)i << 16;
+        else v[mu >> 1] = (uint32_t)i;
+    }
+    __device__ __forceinline__ int get(int mu) const {
+        return (int)(kPack ? (v[mu >> 1] >> (16 * (mu & 1))) & 0xffffu : v[mu]);
+    }
+};
+
 // ---------------------------------------------------------------------------
-// One sample, FP32 path (a1-a3): x[], idx[], J = Jm 2^Je, f.
+// One sample, FP32 path (a1-a3): x[], idx, J = Jm 2^Je, f.
 // ---------------------------------------------------------------------------
-template <int DMAX, bool EXACT, int KIND, bool KP, bool AX>
-__device__ __forceinline__ void point32(const Loop &L, const Strata *S, const float *prm,
+template <int DMAX, bool EXACT, int KIND, bool KP, bool AX, class LT>
+__device__ __forceinline__ void point32(const LT &L, const Strata *S, const float *prm,
                                         uint32_t h, uint32_t j,
                                         const float (&kc)[DMAX], float (&x)[DMAX],
-                                        int (&idx)[DMAX], float &Jm, int &Je, float &f,
+                                        Idx<DMAX> &idx, float &Jm, int &Je, float &f,
                                         int &fe) {
     const int dim = EXACT ? DMAX : L.dim;
     const uint32_t calls = EXACT ? (uint32_t)((DMAX + 3) / 4) : L.calls;
@@ -502,7 +537,7 @@ __device__ __forceinline__ void point32(const Loop &L, const Strata *S, const fl
     for (int q = 0; q < (DMAX + 3) / 4; ++q) {
         if (q < (int)calls) {
             U4 c = {j * calls + (uint32_t)q, h, L.t, L.iid};
-            const U4 r = philox_rk(c, L.rk0, L.rk1);
+            const U4 r = philox_rk(c, L);
 #pragma unroll
             for (int l = 0; l < 4; ++l) {
                 const int mu = 4 * q + l;
@@ -521,7 +556,7 @@ __device__ __forceinline__ void point32(const Loop &L, const Strata *S, const fl
                     const float2 ed = __ldg(L.tab + mu * L.n_g + i);  // {x_i, dx_i}
                     x[mu] = fmaf(ed.y, delta, ed.x);
                     J *= ed.y;
-                    idx[mu] = i;
+                    idx.set(mu, i);
                 }
             }
             renorm(J, e);
@@ -558,8 +593,8 @@ __device__ __forceinline__ void point32(const Loop &L, const Strata *S, const fl
 // increment indices are kept two to a register for the histogram sums.
 // Fewer live registers, so more warps per SM.
 // ---------------------------------------------------------------------------
-template <int DMAX, int KIND, int HM>
-__device__ __forceinline__ void point32_p1(const Loop &L, const Strata *S, const float *kp,
+template <int DMAX, int KIND, int HM, class LT>
+__device__ __forceinline__ void point32_p1(const LT &L, const Strata *S, const float *kp,
                                            uint32_t h, uint32_t j, const float (&kc)[DMAX],
                                            uint32_t (&ip)[DMAX / 2], float &Jm, int &Je,
                                            float &f, uint32_t *hc, uint32_t *HC) {
@@ -570,7 +605,7 @@ __device__ __forceinline__ void point32_p1(const Loop &L, const Strata *S, const
 #pragma unroll
     for (int q = 0; q < (DMAX + 3) / 4; ++q) {
         U4 c = {j * calls + (uint32_t)q, h, L.t, L.iid};
-        const U4 r = philox_rk(c, L.rk0, L.rk1);
+        const U4 r = philox_rk(c, L);
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
             const int mu = 4 * q + l;
@@ -638,8 +673,8 @@ __device__ __forceinline__ double div_by(double a, double n, double rn) {
     return __fma_rn(__fma_rn(-n, q, a), rn, q);
 }
 
-template <int DMAX, int KIND, bool AX>
-__device__ __forceinline__ void point64(const Loop &L, const Strata *S, const double *prm,
+template <int DMAX, int KIND, bool AX, class LT>
+__device__ __forceinline__ void point64(const LT &L, const Strata *S, const double *prm,
                                         uint32_t h, uint32_t j,
                                         const uint32_t (&kd)[DMAX], double (&x)[DMAX],
                                         int (&idx)[DMAX], double &J, double &f) {
@@ -648,7 +683,7 @@ __device__ __forceinline__ void point64(const Loop &L, const Strata *S, const do
     for (int q = 0; q < (DMAX + 3) / 4; ++q) {
         if (q < (int)L.calls) {
             U4 c = {j * L.calls + (uint32_t)q, h, L.t, L.iid};
-            const U4 r = philox_rk(c, L.rk0, L.rk1);
+            const U4 r = philox_rk(c, L);
 #pragma unroll
             for (int l = 0; l < 4; ++l) {
                 const int mu = 4 * q + l;
@@ -691,7 +726,7 @@ __device__ __forceinline__ uint32_t div_nst(uint32_t h, uint32_t magic, int shif
 
 // Mixed-radix digits of h: k_mu = (h / prod_{nu < mu} s_nu) mod s_mu.
 template <int DMAX, bool AX>
-__device__ __forceinline__ void decode_digits(uint32_t h, const Loop &L, const Strata *S, int dim,
+__device__ __forceinline__ void decode_digits(uint32_t h, const LoopBase &L, const Strata *S, int dim,
                                               uint32_t (&kd)[DMAX]) {
 #pragma unroll
     for (int mu = 0; mu < DMAX; ++mu) {
@@ -708,7 +743,7 @@ __device__ __forceinline__ void decode_digits(uint32_t h, const Loop &L, const S
 
 // h -> h + 1 on the digits (carry propagation).
 template <int DMAX, bool AX>
-__device__ __forceinline__ void next_digits(const Loop &L, const Strata *S, int dim,
+__device__ __forceinline__ void next_digits(const LoopBase &L, const Strata *S, int dim,
                                             uint32_t (&kd)[DMAX]) {
     bool carry = true;
 #pragma unroll
@@ -1007,8 +1042,8 @@ __device__ __forceinline__ void MAcc<true>::flush(const SampleOne &a, double *p1
 // each axis is formed, no digit array kept: the digits of the next hypercube
 // are decoded from its index)
 template <int DMAX, bool EXACT, bool F64, int KIND, bool KP, int HM, bool AX, bool MO,
-          bool P1 = false>
-__device__ __forceinline__ void run_samples_t(const Loop &L, const Strata *S, const Ptrs &P,
+          bool P1 = false, class LT>
+__device__ __forceinline__ void run_samples_t(const LT &L, const Strata *S, const Ptrs &P,
                                               const SampleOne *A, double *X1, double *X2,
                                               const void *prm,
                                               uint64_t s_begin, uint64_t s_end, uint64_t h,
@@ -1021,9 +1056,11 @@ __device__ __forceinline__ void run_samples_t(const Loop &L, const Strata *S, co
     typedef typename Real<F64>::T T;
     const int dim = EXACT ? DMAX : L.dim;
     uint32_t j = (uint32_t)(s_begin - lo_off);
-    uint32_t kd[P1 ? 1 : DMAX];
+    // (no digit array kept: P1, and FP32 above D = 12, where registers are short)
+    constexpr bool kDecode = P1 || (!F64 && DMAX > 12);
+    uint32_t kd[kDecode ? 1 : DMAX];
     float kc[DMAX];
-    if constexpr (P1) {
+    if constexpr (kDecode) {
         uint32_t kd1[DMAX];
         decode_digits<DMAX, AX>((uint32_t)h, L, S, dim, kd1);
         hcube_offsets<DMAX, AX>(L, S, kd1, kc);
@@ -1073,7 +1110,7 @@ __device__ __forceinline__ void run_samples_t(const Loop &L, const Strata *S, co
                 hw32 = __frcp_rn((float)nh_cur);
             }
             j = 0;
-            if constexpr (P1) {
+            if constexpr (kDecode) {
                 uint32_t kd1[DMAX];
                 decode_digits<DMAX, AX>((uint32_t)h, L, S, dim, kd1);
                 hcube_offsets<DMAX, AX>(L, S, kd1, kc);
@@ -1083,7 +1120,7 @@ __device__ __forceinline__ void run_samples_t(const Loop &L, const Strata *S, co
             }
         }
         --to_next;
-        int idx[P1 ? 1 : DMAX];
+        typename std::conditional<F64, int[DMAX], Idx<P1 ? 1 : DMAX>>::type idx;
         uint32_t ip[P1 ? DMAX / 2 : 1];  // (P1: increment indices, two to a register)
         T v;
         // FP32: v = J f 2^sexp in [2^-60, 2^60) is summed as is, tiny v in
@@ -1168,7 +1205,8 @@ __device__ __forceinline__ void run_samples_t(const Loop &L, const Strata *S, co
 #pragma unroll
         for (int mu = 0; mu < DMAX; ++mu) {
             if constexpr (P1) bin[mu] = mu * L.n_g + (int)((ip[mu >> 1] >> (16 * (mu & 1))) & 0xffffu);
-            else bin[mu] = mu * L.n_g + idx[mu];
+            else if constexpr (F64) bin[mu] = mu * L.n_g + idx[mu];
+            else bin[mu] = mu < dim ? mu * L.n_g + idx.get(mu) : 0;
         }
         if (big) {
 #pragma unroll
@@ -1230,8 +1268,8 @@ __device__ __forceinline__ void warp_flush(const Ptrs &P, RunTail<F64> t, int la
 }
 
 template <int DMAX, bool EXACT, bool F64, int KIND, bool KP, bool AX, bool MO = false,
-          bool P1 = false>
-__device__ __forceinline__ void run_samples(const Loop &L, const Strata *S, const Ptrs &P,
+          bool P1 = false, class LT>
+__device__ __forceinline__ void run_samples(const LT &L, const Strata *S, const Ptrs &P,
                                             const void *prm, uint64_t s_begin, uint64_t s_end,
                                             uint64_t h, uint64_t lo_off, uint64_t next,
                                             typename Real<F64>::T *hs, float *hs_t, uint32_t *hc,
@@ -1506,15 +1544,48 @@ __global__ void __launch_bounds__(one_max_threads(DMAX, F64, P1), 1)
 // pulls tasks (an integral and a range of `task` samples, big integrals
 // first) and its warps pull warp chunks of the task from a shared counter; the
 // CTA's histograms are flushed when it moves to another integral.
+// Bound: latency.  What limits it is warps per SM, hence registers: the
+// integral's constants, pointers and round keys live in shared memory, the
+// sample loop is compiled for the integral's own dimension, and the FP32 peaks
+// up to D = 12 take one CTA of 768 threads per SM.  512 integrals of 2 to 12
+// dimensions (N_ev 1e4 to 1e6, 15 iterations): 169 ms with everything in
+// registers, two CTAs of 256 (spilling) and one guarded loop; 155 with shared
+// constants; 141 with 768 threads; 124 with a loop per dimension (129 with
+// 1024 threads).
 // ---------------------------------------------------------------------------
 // (AX: the strata per axis from each integral's descriptor, for sets with
 // integrals whose strata differ between axes, §3.2; a separate instantiation
 // so that the other sets keep the one count in registers)
+// The sample loop for the member's own dimension, one instantiation per D up
+// to DMAX (the same operations as the guarded loop, which tests every axis up
+// to DMAX against the dimension).
+template <int D, int DMAX, int KIND>
+__device__ __forceinline__ void run_of_dim(const LoopS &L, const Ptrs &P, const void *prm,
+                                           uint64_t s0, uint64_t s1, uint64_t h, uint64_t lo_off,
+                                           uint64_t hi_off, float *hs, float *hs_t, uint32_t *hc,
+                                           int sexp) {
+    if (L.dim == D)
+        run_samples_t<D, true, false, KIND, false, kHistShared, false, false>(
+            L, nullptr, P, nullptr, nullptr, nullptr, prm, s0, s1, h, lo_off, hi_off, hs, hs_t, hc,
+            sexp, nullptr);
+    else if constexpr (D < DMAX)
+        run_of_dim<D + 1, DMAX, KIND>(L, P, prm, s0, s1, h, lo_off, hi_off, hs, hs_t, hc, sexp);
+}
+
+// Largest CTA of the task kernel, which sets its registers: 768 threads (80
+// registers) for the FP32 peaks up to D = 12, else 256 twice (128 registers).
+__host__ __device__ constexpr int many_max_threads(int dmax, bool f64, int kind) {
+    return !f64 && kind != VP_POSTERIOR && dmax <= 12 ? 768 : 256;
+}
+
 template <int DMAX, bool EXACT, bool F64, int KIND, bool AX = false>
-__global__ void __launch_bounds__(256, 2) k_sample_many(SampleArgs a) {
+__global__ void __launch_bounds__(many_max_threads(DMAX, F64, KIND), many_max_threads(DMAX, F64, KIND) > 256 ? 1 : 2)
+    k_sample_many(SampleArgs a) {
     typedef typename Real<F64>::T T;
+    constexpr bool kOwnDim = many_max_threads(DMAX, F64, KIND) > 256 && !EXACT && !AX;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_task, s_wc;
+    __shared__ uint4 s_keys[5];
     float *sprm = (float *)smem;
     // histograms: sums (FP64, or FP32 and the FP32 tiny sums), then counts
     T *hs = (T *)(smem + (size_t)a.prm_words * 4);
@@ -1524,14 +1595,21 @@ __global__ void __launch_bounds__(256, 2) k_sample_many(SampleArgs a) {
     const uint32_t wchunk = 32u * (uint32_t)a.r;
     pdl_wait();
 
+    // the integral's constants and pointers, in shared memory: broadcast loads
+    // where they are used, not registers held across the sample loop
+    __shared__ LoopS s_loop;
+    __shared__ Ptrs s_ptrs;
+    __shared__ int s_sexp;
+    __shared__ const void *s_prm;
+    __shared__ const Strata *s_strata;
+    const LoopS &L = s_loop;
+    const Ptrs &P = s_ptrs;
     int cur = -1;
-    Loop L;
-    Ptrs P;
-    const void *prm = nullptr;
-    int bins = 0, sexp = 0;
-    const Strata *S = nullptr;
 
     auto flush_hist = [&]() {
+        const int bins = L.dim * L.n_g, sexp = s_sexp;
+        double *const HS = P.HS;
+        uint32_t *const HC = P.HC;
         // each CTA starts at its own bin (in whole warps), so that the CTAs'
         // global reductions do not all queue on the same addresses at once
         const int rot = (int)(((uint32_t)blockIdx.x * (uint32_t)bins / gridDim.x) & ~31u);
@@ -1541,39 +1619,48 @@ __global__ void __launch_bounds__(256, 2) k_sample_many(SampleArgs a) {
             if (n) {
                 double d = F64 ? (double)hs[b] * pow2d(-2 * sexp) : f2d_pow2((float)hs[b], -2 * sexp);
                 if (!F64 && hs_t[b] != 0.0f) d += f2d_pow2(hs_t[b], -2 * (sexp + kTinyShift));
-                red_add(P.HS + b, d);
-                red_add(P.HC + b, n);
+                red_add(HS + b, d);
+                red_add(HC + b, n);
             }
         }
     };
-    auto enter = [&](int g) {  // all threads; caller synchronises afterwards
+    auto enter = [&](int g) {  // all threads; caller synchronises before (after a flush) and afterwards
         cur = g;
         const Desc *dp = a.desc + __ldg(a.members + g);
-        State *st = (State *)__ldg((const unsigned long long *)&dp->st);
-        const uint32_t t_it = __ldcg(&st->t);
-        if (threadIdx.x == 0)  // every CTA of the integral writes the same
+        if (threadIdx.x == 0) {
+            State *st = (State *)__ldg((const unsigned long long *)&dp->st);
+            const uint32_t t_it = __ldcg(&st->t);
+            // every CTA of the integral writes the same
             st->hist_par = (t_it & 1u) | (__ldg(&dp->d_weighted) ? 2u : 0u);
-        L = make_loop(dp, t_it);
-        if (AX) S = &dp->strata;
-        sexp = F64 ? 0 : __ldcg(&st->scale_exp);  // (FP64: unscaled, as in k_sample_one)
-        bins = L.dim * L.n_g;
-        P.off = (const uint64_t *)__ldg((const unsigned long long *)&dp->off);
-        P.nh = (const uint32_t *)__ldg((const unsigned long long *)&dp->n_h);
-        P.n_hc = __ldg(&dp->n_hc);
-        P.n_total = __ldcg(P.off + P.n_hc);
-        // accumulators of this iteration: buffer (t & 1) of the double-buffered pairs
-        const uint64_t par = t_it & 1u;
-        P.S1 = (double *)__ldg((const unsigned long long *)&dp->s1) + par * P.n_hc;
-        P.S2 = (double *)__ldg((const unsigned long long *)&dp->s2) + par * P.n_hc;
-        P.HS = (double *)__ldg((const unsigned long long *)&dp->hsum) + par * bins;
-        P.HC = (uint32_t *)__ldg((const unsigned long long *)&dp->hcnt) + par * bins;
-        if (F64) {
-            prm = (const void *)__ldg((const unsigned long long *)&dp->prm);
-        } else {
-            load_prm32(dp, sprm, a.prm_words);
-            prm = (const void *)sprm;
+            *(LoopBase *)&s_loop = make_base(dp, t_it);
+            s_loop.keys = s_keys;
+            s_strata = &dp->strata;
+            s_sexp = F64 ? 0 : __ldcg(&st->scale_exp);  // (FP64: unscaled, as in k_sample_one)
+            const uint64_t n_hc = __ldg(&dp->n_hc);
+            const uint64_t bins = (uint64_t)(__ldg(&dp->dim) * __ldg(&dp->n_g));
+            Ptrs q;
+            q.off = (const uint64_t *)__ldg((const unsigned long long *)&dp->off);
+            q.nh = (const uint32_t *)__ldg((const unsigned long long *)&dp->n_h);
+            q.n_hc = n_hc;
+            q.n_total = __ldcg(q.off + n_hc);
+            // accumulators of this iteration: buffer (t & 1) of the double-buffered pairs
+            const uint64_t par = t_it & 1u;
+            q.S1 = (double *)__ldg((const unsigned long long *)&dp->s1) + par * n_hc;
+            q.S2 = (double *)__ldg((const unsigned long long *)&dp->s2) + par * n_hc;
+            q.HS = (double *)__ldg((const unsigned long long *)&dp->hsum) + par * bins;
+            q.HC = (uint32_t *)__ldg((const unsigned long long *)&dp->hcnt) + par * bins;
+            s_ptrs = q;
+            s_prm = F64 ? (const void *)__ldg((const unsigned long long *)&dp->prm) : (const void *)sprm;
         }
+        if (threadIdx.x >= 32 && threadIdx.x < 37) {
+            const uint32_t i = threadIdx.x - 32u, r = 2u * i;
+            const uint32_t k0 = __ldg(&dp->key0) + r * 0x9E3779B9u;
+            const uint32_t k1 = __ldg(&dp->key1) + r * 0xBB67AE85u;
+            s_keys[i] = make_uint4(k0, k1, k0 + 0x9E3779B9u, k1 + 0xBB67AE85u);
+        }
+        if (!F64) load_prm32(dp, sprm, a.prm_words);
         if (a.hist_shared) {
+            const int bins = __ldg(&dp->dim) * __ldg(&dp->n_g);
             for (int b = threadIdx.x; b < bins; b += blockDim.x) {
                 hs[b] = (T)0;
                 if (!F64) hs_t[b] = 0.0f;
@@ -1616,10 +1703,17 @@ __global__ void __launch_bounds__(256, 2) k_sample_many(SampleArgs a) {
             uint64_t lo_off = 0, hi_off = 0;
             const uint64_t h =
                 lane_find_hcube(P.off, P.n_hc, hb, s0, s0 < s1, lane, &lo_off, &hi_off);
-            if (s0 < s1)
-                run_samples<DMAX, EXACT, F64, KIND, false, AX>(
-                    L, S, P, prm, s0, s1, h, lo_off, hi_off, hs, hs_t, hc,
-                    a.hist_shared ? kHistShared : kHistGlobal, sexp);
+            if (s0 < s1) {
+                if (kOwnDim && a.hist_shared) {
+                    if constexpr (kOwnDim)
+                        run_of_dim<1, DMAX, KIND>(L, P, s_prm, s0, s1, h, lo_off, hi_off, hs, hs_t,
+                                                  hc, s_sexp);
+                } else {
+                    run_samples<DMAX, EXACT, F64, KIND, false, AX>(
+                        L, s_strata, P, s_prm, s0, s1, h, lo_off, hi_off, hs, hs_t, hc,
+                        a.hist_shared ? kHistShared : kHistGlobal, s_sexp);
+                }
+            }
         }
     }
     if (cur >= 0 && a.hist_shared) flush_hist();
@@ -1662,8 +1756,11 @@ __global__ void k_eval(const Desc *desc, int member, int64_t n, const uint64_t *
             int Je;
             hcube_offsets<DMAX, true>(L, S, kd, kc);
             int fe;
-            point32<DMAX, EXACT, KIND, false, true>(L, S, sprm, (uint32_t)hs[k], js[k], kc, x, idx,
+            Idx<DMAX> ix;
+            point32<DMAX, EXACT, KIND, false, true>(L, S, sprm, (uint32_t)hs[k], js[k], kc, x, ix,
                                                     Jm, Je, ff, fe);
+#pragma unroll
+            for (int mu = 0; mu < DMAX; ++mu) idx[mu] = mu < dim ? ix.get(mu) : 0;
 #pragma unroll
             for (int mu = 0; mu < DMAX; ++mu) xd[mu] = (double)x[mu];
             jac = ldexp((double)Jm, Je);

@@ -775,9 +775,10 @@ def run_ours(args):
                             "final result, wall clock" % args.steps},
             "roofline": roof, "clocks": clocks,
             "chain": _chain_view(g.n_hc, prob.dim, prob.n_g, peaks.get("hbm_gbs", 6800.0)),
-            # sample, estimate, alloc, offsets, refine (+ the task prefix for the task
-            # kernel, + the several-outputs estimate)
-            "gpu_launches": (5 + (g.tuning()["scheme"] == "tasks") + bayes) * args.steps,
+            # sample, estimate, alloc, offsets, refine (sample, adapt, refine up to 4096
+            # hypercubes) + the task prefix for the task kernel, + the several-outputs
+            # estimate
+            "gpu_launches": ((5 if g.n_hc > 4096 else 3) + (g.tuning()["scheme"] == "tasks") + bayes) * args.steps,
             "sample_launch": g.tuning(),
             "integral": dict(_integral(g, prob, ball, late_half=expo), exact=prob.exact)}
     if bayes:

@@ -766,7 +766,8 @@ __global__ void __launch_bounds__(kSubH, 4) k_offsets_wide(const Desc *desc,
 // terms 4t + q of block k, as k_estimate does (the same sums in the same
 // order), every CTA adds the block sums itself, allocates n_h of its
 // hypercubes from the d_h it still holds, then takes the quarter q of block k
-// in order for the offsets.
+// in order for the offsets.  11.5 us against 8.7 + 7.1 + 5.2; 16 steps of 1e4
+// samples 721 -> 582 us.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_adapt_small(const Desc *desc) {
     namespace cg = cooperative_groups;
@@ -870,7 +871,8 @@ __global__ void __launch_bounds__(256) k_adapt_small(const Desc *desc) {
 // One axis is latency-bound (~14 us); many (a batch, a server's requests) are
 // bound by the FP64 pipe, 16 cycles per warp instruction, so what every thread
 // needs of the cluster (1 / sum, the bases, the step) is formed by one warp,
-// and the searches compare the bits of their nonnegative numbers.
+// and the searches compare the bits of their nonnegative numbers (256 requests,
+// 2136 axes: 54.4 -> 50.0 ms for 24 iterations).
 // ---------------------------------------------------------------------------
 constexpr int kRefineCtas = 8;
 constexpr int kRefineThreads = 128;

@@ -180,7 +180,8 @@ __device__ __forceinline__ float f_peaks32_param(const float *kp, int K, int dim
 // would be the same for every point and add up), and six more operations.
 // The points are visited group by group, so that each weight's two factors
 // are formed once.  Returns the same value up to rounding as the sum of
-// logarithms, and the same zeros, infinities and NaN.
+// logarithms, and the same zeros, infinities and NaN.  (With k_estimate_multi:
+// 15 iterations of 1e5 samples, 50 points, 8 outputs, 30.6 -> 11.4 ms.)
 // After the blob: {fast, 1/(2 sy^2) hi, lo, 1/(200 sy^2) hi, lo} (fast 0:
 // those reciprocals are out of range, the kernel divides).
 __device__ __forceinline__ double mul2(double a, double hi, double lo) {
@@ -646,7 +647,8 @@ __device__ __forceinline__ void point32_p1(const LT &L, const Strata *S, const f
 // per warp instruction), so the steps are formed with as few FP64 instructions
 // as give the same bits: k + u by one subtraction, y by three operations
 // instead of a division, the increment by a round-down addition instead of a
-// floor and two conversions.
+// floor and two conversions (8-D, four peaks, 1e6 samples: 0.87 -> 0.77 ms a
+// step; 0.70 with the fused distances of f_peaks64).
 // ---------------------------------------------------------------------------
 // k + u with u = (w + 1/2) 2^-32.  Up to 2^19 strata the sum has at most 52
 // bits, so it is exact: its bits are put below the leading bit of 2^19 (unit
@@ -1438,7 +1440,8 @@ __global__ void __launch_bounds__(one_max_threads(DMAX, F64, P1), 1)
         // same whatever their lanes do, paid for all 32.  (FP64 up to 8 samples
         // per lane: beyond it the idle lanes cost less than a warp in nine.
         // FP32 at one per lane, up to D = 8 and not in parts: its sums depend on
-        // which samples a lane, a warp's combine and a CTA's histogram add.)
+        // which samples a lane, a warp's combine and a CTA's histogram add.  A 4-D
+        // FP64 job of 1e4 samples: 1104 -> 940 us.)
         uint32_t Ws = W, ws = w;
         if constexpr (F64 || DMAX <= 8) {
             const uint32_t rounds = n_st / (32u * W) + (n_st % (32u * W) != 0u ? 1u : 0u);

@@ -215,8 +215,11 @@ vp_status vp_step_read_flush(vp_ctx *ctx, int *have, double *i_j, double *var_j)
  * Identical sums give identical estimates, allocations and grids on every
  * rank.  FP32 peak families with more than 8 peaks, and contexts with extra
  * outputs, are refused (VP_EINVAL).  vp_iterate_part may be called for
- * several parts on one context (they add up).  Buffers are the caller's;
- * nothing is allocated. */
+ * several parts on one context (they add up).  The launch shape of a part of
+ * an FP32 integral follows from its sizes alone (or vp_set_tuning's, if the
+ * caller fixed one), never from a measurement: the FP32 roundings in the
+ * exported sums depend on it.  Buffers are the caller's; nothing is
+ * allocated. */
 vp_status vp_iterate_part(vp_ctx *ctx, int part, int n_parts, void *stream);
 vp_status vp_partials_size(vp_ctx *ctx, int64_t *n);
 vp_status vp_partials_export(vp_ctx *ctx, double *buf, void *stream);

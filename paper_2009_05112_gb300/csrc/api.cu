@@ -1517,6 +1517,61 @@ static vp_status shard_check(vp_ctx *c) {
     return VP_OK;
 }
 
+// Launch shape of a part of an FP32 integral with shared-memory histograms, by
+// rule: a CTA adds its d_i terms in FP32 and a cluster its CTAs' sums, so the
+// shape decides the roundings of the exported sums (16-D, 250,000 samples: 1e-9
+// to 3e-9 of their norm between shapes, a few 1e-10 between runs of one), and a
+// shape picked by a stopwatch would let two runs, or two ranks, differ by them.
+// Pairs of CTAs (half the global reductions of a flush), one CTA of the
+// kernel's largest size per SM.  Peaks up to D = 8: the largest size that gives
+// every lane a sample (7-D, 3e5 samples in 4 parts: 512 threads 100 us, 1024
+// 120); up to D = 3, whose histograms are small, three CTAs of 256 (2-D, 3e5
+// samples: 62 us, 1024 threads 68).  Large parts with the dynamic tail where it
+// gains (8-D, 5e7 samples: 1642 us, without it 1707; 20-D ball: 2290, 2165),
+// its sums' roundings then by the order in which the warps pull.  Posteriors
+// above D = 8 keep the planned shape (the autotuner picks the task kernel there,
+// which has no parts).  Otherwise no slower than the autotuner's picks but by
+// their own scatter.
+static bool part_shape(const Set &s, Group &g, int n_parts, Group::Shape *out) {
+    const Member &mb = s.m[g.members[0]];
+    const double expect = (double)mb.p.n_ev + 2.0 * (double)mb.n_hc;
+    if (g.fixed || g.prec != VP_FP32 || !g.hist_one || expect < kTuneMinSamples) return false;
+    const bool peaks = g.kind != VP_POSTERIOR;
+    const int dim = mb.p.dim;
+    if (!peaks && dim > 8) {
+        out->threads = g.threads_plan;
+        out->blocks = g.blocks_plan;
+        out->cs = g.cs_plan;
+        return true;
+    }
+    if (!g.part_shapes_known) {
+        for (Group::Shape &q : g.part_shape) {
+            if (q.threads > one_max_threads(bucket_dim(g.bucket), false, g.p1)) continue;
+            if (sample_occupancy_f32(g.bucket, g.exact, g.kind, true, q.threads, g.smem_one, false,
+                                     g.p1) < q.per_sm)
+                continue;
+            q.blocks = q.per_sm * s.n_sm;
+            if (q.blocks % 2 == 0 &&
+                sample_cluster_ctas_f32(g.bucket, g.exact, g.kind, 2, q.blocks, q.threads,
+                                        g.smem_one, g.p1) >= q.blocks)
+                q.cs = 2;
+        }
+        g.part_shapes_known = true;
+    }
+    const double share = (double)mb.p.n_ev / n_parts;
+    const Group::Shape *best = nullptr;
+    for (const Group::Shape &q : g.part_shape) {  // (ascending sizes)
+        if (!q.blocks || (q.threads == 256 && !(peaks && dim <= 3))) continue;
+        const bool full = share >= (double)s.n_sm * q.threads;
+        if (!best || !(peaks && dim <= 8) || (best->threads != 256 && full)) best = &q;
+    }
+    if (!best) return false;
+    *out = *best;
+    out->static16 = share >= (dim <= 8 ? kTailMinSamples : 4.0 * kTailMinSamples) ? kTailShare
+                                                                                  : kStaticShare;
+    return true;
+}
+
 extern "C" vp_status vp_iterate_part(vp_ctx *c, int part, int n_parts, void *stream) {
     vp_status st = shard_check(c);
     if (st != VP_OK) return st;
@@ -1525,16 +1580,25 @@ extern "C" vp_status vp_iterate_part(vp_ctx *c, int part, int n_parts, void *str
     NvtxRange nv("vp.iterate_part");
     Set &s = c->set;
     cudaStream_t strm = (cudaStream_t)stream;
+    Group::Shape shape{};
+    const bool ruled = part_shape(s, s.groups[0], n_parts, &shape);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     CU(cudaStreamIsCapturing(strm, &cap));
-    if (cap != cudaStreamCaptureStatusActive) {
+    if (cap != cudaStreamCaptureStatusActive && !ruled) {
         st = tune(s, strm);
         if (st != VP_OK) return st;
     }
-    // the one-integral kernel in its tuned shape, or its planned one if the
-    // tuner chose the task kernel (which has no sample ranges)
+    // the one-integral kernel in the shape of the rule, else its tuned one, or
+    // its planned one if the tuner chose the task kernel (which has no sample
+    // ranges)
     Group g = s.groups[0];
-    if (!g.one) {
+    if (ruled) {
+        g.one = true;
+        g.blocks = shape.blocks;
+        g.cs = shape.cs;
+        g.threads_one = shape.threads;
+        g.args1.static16 = shape.static16;
+    } else if (!g.one) {
         g.one = true;
         g.blocks = g.blocks_plan;
         g.cs = g.cs_plan;
@@ -2267,6 +2331,7 @@ extern "C" vp_status vp_set_tuning(vp_ctx *c, int scheme, int blocks, int thread
     g.threads_one = threads;
     g.static16 = static16;
     g.tuned_final = true;
+    g.fixed = true;
     g.args1.r = run;
     g.args1.static16 = static16;
     double expect = 0.0;

@@ -111,6 +111,13 @@ struct Group {
     // the one-integral kernel's shape as planned (before the autotuner), for
     // launches that need that kernel whatever the tuner chose (sharded sampling)
     int blocks_plan = 0, cs_plan = 1, threads_plan = 256;
+    bool fixed = false;  // the caller fixed the launch shape (vp_set_tuning)
+    // the one-integral kernel's candidate shapes for parts (blocks 0: not resident)
+    struct Shape {
+        int threads, per_sm, blocks = 0, cs = 1, static16 = kStaticShare;
+    };
+    Shape part_shape[4] = {{256, 3}, {512, 1}, {768, 1}, {1024, 1}};
+    bool part_shapes_known = false;
     // histograms of the one-integral kernel (one CTA per SM fits more shared
     // memory than the task kernel's two): kHist* mode and dynamic shared bytes
     int hist_one = 0;

@@ -216,9 +216,11 @@ __device__ __forceinline__ double f_post64(const double *p, int dim, const doubl
             }
             const double r = y[i] - model;
             double r2 = -r * r;
-            // (beyond 2^664 both exponentials are zero; the pair's low product
-            // must not overflow)
-            if ((uint32_t)(__double2hiint(r2) & 0x7fffffff) - 0x69700000u <= 0x7ff00000u - 0x69700000u &&
+            // (with reciprocals, 200 sy^2 < 2^400: beyond 2^664 both exponentials
+            // are zero, and the pair's low product must not overflow; the
+            // divisions take r2 as it is, a wide noise's terms are not zero there)
+            if (fast &&
+                (uint32_t)(__double2hiint(r2) & 0x7fffffff) - 0x69700000u <= 0x7ff00000u - 0x69700000u &&
                 !isnan(r2))
                 r2 = -pow2d(664);
             const double en = exp(fast ? mul2(r2, nh, nl) : r2 / (2.0 * sy * sy));

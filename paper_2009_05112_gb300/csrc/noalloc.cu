@@ -92,7 +92,8 @@ __global__ void __launch_bounds__(256) ks_sum(const double *d_h, uint64_t n_hc, 
 }
 
 // The reading's quotient as written, for sums so large that N_ev d_h may
-// overflow (a call, so that its FP64 work stays out of the common path).
+// overflow and for d_h outside [0, sum d] (a call, so that its FP64 work stays
+// out of the common path).
 __device__ __noinline__ uint32_t alloc_literal(double dh, double n_ev_d, double sum_d, int plus2) {
     const double q = __ddiv_rn(__dmul_rn(n_ev_d, dh), sum_d);
     double fl = floor(q);
@@ -144,7 +145,12 @@ __global__ void __launch_bounds__(256) ks_alloc(const double *d_h, uint64_t n_hc
     K.n_hc = n_hc;
     K.plus2 = plus2 != 0;
     if (!vp::finite_bits(K.sum_d)) return;  // allocation left unchanged
-    const bool huge = !vp::finite_bits(n_ev_d * K.sum_d);
+    // d_h whose bits pass `lit` take the quotient as written: all but zero where
+    // N_ev d_h may overflow, else a negative one or one above the sum (outside
+    // the documented range; none where sum d is not positive)
+    const uint64_t sum_bits = (uint64_t)__double_as_longlong(K.sum_d);
+    const uint64_t lit = (int64_t)sum_bits <= 0 ? ~0ull
+                         : vp::finite_bits(n_ev_d * K.sum_d) ? sum_bits : 0ull;
     const uint64_t h0 = (uint64_t)blockIdx.x * 1024 + 4u * threadIdx.x;
     const bool full = h0 + 4 <= n_hc;
     double dh[4];
@@ -161,7 +167,9 @@ __global__ void __launch_bounds__(256) ks_alloc(const double *d_h, uint64_t n_hc
     for (int q = 0; q < 4; ++q) {
         n[q] = 0u;
         if (h0 + q < n_hc)
-            n[q] = huge ? alloc_literal(dh[q], n_ev_d, K.sum_d, plus2) : vp::alloc_one(dh[q], K, 0);
+            n[q] = (uint64_t)__double_as_longlong(dh[q]) > lit
+                       ? alloc_literal(dh[q], n_ev_d, K.sum_d, plus2)
+                       : vp::alloc_one(dh[q], K, 0);
         own += n[q];
     }
     if (VEC && full) {

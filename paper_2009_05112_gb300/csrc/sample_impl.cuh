@@ -274,7 +274,10 @@ __device__ __forceinline__ double f_post64(const double *p, int dim, const doubl
 // Bound: the three MUFU operations of a point (6 cycles of an SM per warp and
 // point).  A line (P = 2) reads a point as one 16-byte shared load and takes
 // two multiply-adds; testing every m < DMAX against P, as the general form
-// once did here too, cost ~100 cycles per warp and point at D = 21.
+// once did here too, cost ~100 cycles per warp and point at D = 21.  The
+// general form reads four numbers and tests once a group of four whether any is
+// left (a branch per m, 16-D and P = 12 at 1e6: 352 us a step; a test per m 224;
+// this 227, and 21-D, P = 20: 529, 1176, 387).
 template <int DMAX, bool LINE>
 __device__ __forceinline__ float post32_points(const float *p, int n, int npar, int ngrp,
                                                const float (&x)[DMAX]) {
@@ -296,12 +299,20 @@ __device__ __forceinline__ float post32_points(const float *p, int n, int npar, 
                 y = v.x;
                 model = fmaf(v.z, x[1], v.y * x[0]);
             } else {
-                y = q[0];
-                model = 0.0f;
+                // {y, A[0], A[1], A[2]}, then four of A at a time
+                const float4 v = *(const float4 *)q;
+                y = v.x;
+                model = v.y * x[0];
+                if (DMAX > 1 && npar > 1) model = fmaf(v.z, x[1], model);
+                if (DMAX > 2 && npar > 2) model = fmaf(v.w, x[2], model);
 #pragma unroll
-                for (int m = 0; m < DMAX; ++m) {
+                for (int m = 3; m < DMAX; m += 4) {
                     if (m >= npar) break;
-                    model = fmaf(q[1 + m], x[m], model);
+                    const float4 a = *(const float4 *)(q + 1 + m);
+                    model = fmaf(a.x, x[m], model);
+                    if (m + 1 < DMAX && m + 1 < npar) model = fmaf(a.y, x[m + 1], model);
+                    if (m + 2 < DMAX && m + 2 < npar) model = fmaf(a.z, x[m + 2], model);
+                    if (m + 3 < DMAX && m + 3 < npar) model = fmaf(a.w, x[m + 3], model);
                 }
             }
             const float r = y - model;

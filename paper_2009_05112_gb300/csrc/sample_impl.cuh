@@ -518,30 +518,29 @@ __device__ __forceinline__ void hcube_offsets(const LoopBase &L, const Strata *S
         kc[mu] = ((float)kd[mu] - 0.99999994039535522461f) * c32_of<AX>(L, S, mu);
 }
 
-// Increment indices (below kMaxNg = 4096) of a sample, FP32 path: above D = 12
-// two to a register, which is what keeps the sample loop's arrays of 24 axes
-// out of local memory.
-template <int DMAX> struct Idx {
-    static constexpr bool kPack = DMAX > 12;
-    uint32_t v[kPack ? (DMAX + 1) / 2 : DMAX];
+// Increment indices (below kMaxNg = 4096) of a sample, FP32 path: packed, two to
+// a register, where the sample loop's arrays of so many axes would not stay out
+// of local memory (see run_samples_t).
+template <int DMAX, bool PACK> struct Idx {
+    uint32_t v[PACK ? (DMAX + 1) / 2 : DMAX];
     __device__ __forceinline__ void set(int mu, int i) {
-        if (!kPack) v[mu] = (uint32_t)i;
+        if (!PACK) v[mu] = (uint32_t)i;
         else if (mu & 1) v[mu >> 1] |= (uint32_t)i << 16;
         else v[mu >> 1] = (uint32_t)i;
     }
     __device__ __forceinline__ int get(int mu) const {
-        return (int)(kPack ? (v[mu >> 1] >> (16 * (mu & 1))) & 0xffffu : v[mu]);
+        return (int)(PACK ? (v[mu >> 1] >> (16 * (mu & 1))) & 0xffffu : v[mu]);
     }
 };
 
 // ---------------------------------------------------------------------------
 // One sample, FP32 path (a1-a3): x[], idx, J = Jm 2^Je, f.
 // ---------------------------------------------------------------------------
-template <int DMAX, bool EXACT, int KIND, bool KP, bool AX, class LT>
+template <int DMAX, bool EXACT, int KIND, bool KP, bool AX, bool PACK, class LT>
 __device__ __forceinline__ void point32(const LT &L, const Strata *S, const float *prm,
                                         uint32_t h, uint32_t j,
                                         const float (&kc)[DMAX], float (&x)[DMAX],
-                                        Idx<DMAX> &idx, float &Jm, int &Je, float &f,
+                                        Idx<DMAX, PACK> &idx, float &Jm, int &Je, float &f,
                                         int &fe) {
     const int dim = EXACT ? DMAX : L.dim;
     const uint32_t calls = EXACT ? (uint32_t)((DMAX + 3) / 4) : L.calls;
@@ -1071,8 +1070,17 @@ __device__ __forceinline__ void run_samples_t(const LT &L, const Strata *S, cons
     typedef typename Real<F64>::T T;
     const int dim = EXACT ? DMAX : L.dim;
     uint32_t j = (uint32_t)(s_begin - lo_off);
-    // (no digit array kept: P1, and FP32 above D = 12, where registers are short)
-    constexpr bool kDecode = P1 || (!F64 && DMAX > 12);
+    // FP32 above D = 12 where registers are short (a dimension guard's or the
+    // task kernel's arrays went to local memory): indices two to a register, and
+    // no digit array.  The one-integral kernel's exact dimensions fit as they
+    // are, and were slower this way up to D = 20 (20-D peaks at 1e7 901 us a
+    // step, 812 as they are) and for the ball at 24 (1882 us at 3e7, 1658), not
+    // for what else has 24 (peaks 2513 us, 2651).
+    constexpr bool kOneExact =
+        EXACT && (KP || (KIND == VP_POSTERIOR && std::is_same<LT, Loop>::value));
+    constexpr bool kShort =
+        !F64 && DMAX > 12 && !(kOneExact && (DMAX <= 20 || KIND == VP_BALL));
+    constexpr bool kDecode = P1 || kShort;
     uint32_t kd[kDecode ? 1 : DMAX];
     float kc[DMAX];
     if constexpr (kDecode) {
@@ -1135,7 +1143,7 @@ __device__ __forceinline__ void run_samples_t(const LT &L, const Strata *S, cons
             }
         }
         --to_next;
-        typename std::conditional<F64, int[DMAX], Idx<P1 ? 1 : DMAX>>::type idx;
+        typename std::conditional<F64, int[DMAX], Idx<P1 ? 1 : DMAX, kShort>>::type idx;
         uint32_t ip[P1 ? DMAX / 2 : 1];  // (P1: increment indices, two to a register)
         T v;
         // FP32: v = J f 2^sexp in [2^-60, 2^60) is summed as is, tiny v in
@@ -1162,7 +1170,7 @@ __device__ __forceinline__ void run_samples_t(const LT &L, const Strata *S, cons
             } else {
                 float x[DMAX];
                 int fe;
-                point32<DMAX, EXACT, KIND, KP, AX>(L, S, (const float *)prm, (uint32_t)h, j, kc, x,
+                point32<DMAX, EXACT, KIND, KP, AX, kShort>(L, S, (const float *)prm, (uint32_t)h, j, kc, x,
                                                    idx, Jm, Je, f, fe);
                 Je += fe;  // J f = (Jm f) 2^(Je + fe)
             }
@@ -1772,8 +1780,8 @@ __global__ void k_eval(const Desc *desc, int member, int64_t n, const uint64_t *
             int Je;
             hcube_offsets<DMAX, true>(L, S, kd, kc);
             int fe;
-            Idx<DMAX> ix;
-            point32<DMAX, EXACT, KIND, false, true>(L, S, sprm, (uint32_t)hs[k], js[k], kc, x, ix,
+            Idx<DMAX, false> ix;
+            point32<DMAX, EXACT, KIND, false, true, false>(L, S, sprm, (uint32_t)hs[k], js[k], kc, x, ix,
                                                     Jm, Je, ff, fe);
 #pragma unroll
             for (int mu = 0; mu < DMAX; ++mu) idx[mu] = mu < dim ? ix.get(mu) : 0;

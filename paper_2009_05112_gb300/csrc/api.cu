@@ -515,13 +515,40 @@ static vp_status plan_groups(Set &s) {
     return VP_OK;
 }
 
-// Task-kernel launch shape of a group: shared-memory histograms when the
-// largest member's fit (with the FP32 constants) in 112 KB, two CTAs per SM at
-// most, tasks of ~1/8 of a CTA's share in whole warp chunks.  Groups of
-// several FP32 peak integrals up to D = 12 take one CTA of 768 threads per SM
-// where the histograms fit in 220 KB (see k_sample_many); larger dimensions
-// and posteriors keep 256 (posteriors spill at 80 registers: 256 requests 62.7
-// ms against 50.1).
+// Whether a group's task kernel takes the wide CTA (768 threads, one per SM)
+// instead of two of 256: FP32 peaks up to D = 12, several integrals, shared
+// histograms.  A CTA's warps share one task at a time, and a task, 1/8 of a
+// CTA's share of the samples, has at least 8 warp chunks: below 152 x 8 x 2048
+// samples 24 warps have 8 chunks to share (16 integrals of 2 to 12 dimensions,
+// a step, two CTAs / one wide: 80 / 97 us at 3e4 samples each, 161 / 174 at
+// 1e5, 416 / 305 at 3e5; 4 of 8-D at 1e5: 56 / 74).  Strata per axis, whose
+// loop is not compiled per dimension: from twice that (32 of 5 to 8 dimensions
+// at 1e5: 262 / 291; at 3e5 647 / 585).  Histograms that only one CTA per SM
+// can hold, added in global memory otherwise: from half of it (2 of 12-D,
+// N_g = 1000, at 1e6: 392 / 184).  At most a quarter of the samples on one or
+// two axes, where 24 warps add to few bins of one histogram (4 of 2-D at 3e6:
+// 1210 / 1620), and up to D = 4 four integrals or more (2 of 3-D at 1e6: 145 /
+// 160; 16 at 3e5: 289 / 244).
+constexpr double kWideMinSamples = 2.5e6;
+static bool wide_pays(const std::vector<const Member *> &m, const Group &g, double expect,
+                      size_t hist_bytes, size_t prm_bytes) {
+    if (g.members.size() < 2 || !many_wide(bucket_dim(g.bucket), g.prec == VP_FP64, g.kind) ||
+        hist_bytes + prm_bytes > kOneSmemMax)
+        return false;
+    if (bucket_dim(g.bucket) <= 4 && g.members.size() < 4) return false;
+    double low = 0.0;
+    for (uint32_t i : g.members)
+        if (m[i]->p.dim <= 2) low += (double)m[i]->p.n_ev + 2.0 * (double)m[i]->n_hc;
+    if (low > 0.25 * expect) return false;
+    if (hist_bytes + prm_bytes > kTwoSmemMax) return expect >= 0.5 * kWideMinSamples;
+    return expect >= (g.uniform ? 1.0 : 2.0) * kWideMinSamples;
+}
+
+// Task-kernel launch shape of a group: the wide CTA where it pays, else two CTAs
+// per SM at most, with shared-memory histograms when the largest member's fit
+// (with the FP32 constants) in 112 KB; tasks of ~1/8 of a CTA's share in whole
+// warp chunks.  Larger dimensions and posteriors keep 256 threads (posteriors
+// spill at 80 registers: 256 requests 62.7 ms against 50.1).
 vp_status vp::group_config_many(const std::vector<const Member *> &m, Group &g, int n_sm) {
     double expect = 0.0;
     int max_bins = 0, max_words = 0;
@@ -543,20 +570,19 @@ vp_status vp::group_config_many(const std::vector<const Member *> &m, Group &g, 
     g.hist_words = max_bins;
     g.prm_words = g.prec == VP_FP64 ? 0 : ((max_words + 3) & ~3);
     const size_t prm_bytes = (size_t)g.prm_words * 4;
-    // (one member: the autotuner's task scheme, whose CTAs have 256 threads)
-    const int wide = many_max_threads(bucket_dim(g.bucket), g.prec == VP_FP64, g.kind);
-    if (g.members.size() > 1 && hist_bytes + prm_bytes <= kOneSmemMax) g.threads = wide;
-    g.hist_shared = g.threads > 256 || hist_bytes + prm_bytes <= 112 * 1024 ? 1 : 0;
+    g.wide = wide_pays(m, g, expect, hist_bytes, prm_bytes);
+    if (g.wide) g.threads = kWideThreads;
+    g.hist_shared = g.wide || hist_bytes + prm_bytes <= kTwoSmemMax ? 1 : 0;
     g.smem = prm_bytes + (g.hist_shared ? hist_bytes : 0);
     g.one = false;
     g.cs = 1;
     cudaError_t e = g.prec == VP_FP64
                         ? sample_smem_config_f64(g.bucket, g.exact, g.kind, false, (int)std::max<size_t>(g.smem, 48 * 1024), false, !g.uniform)
-                        : sample_smem_config_f32(g.bucket, g.exact, g.kind, false, (int)std::max<size_t>(g.smem, 48 * 1024), !g.uniform);
+                        : sample_smem_config_f32(g.bucket, g.exact, g.kind, false, (int)std::max<size_t>(g.smem, 48 * 1024), !g.uniform, false, g.wide);
     if (e != cudaSuccess) return fail(VP_ECUDA, "kernel attributes: %s", cudaGetErrorString(e));
     g.occ_many = g.prec == VP_FP64
                      ? sample_occupancy_f64(g.bucket, g.exact, g.kind, false, g.threads, g.smem, false, !g.uniform)
-                     : sample_occupancy_f32(g.bucket, g.exact, g.kind, false, g.threads, g.smem, !g.uniform);
+                     : sample_occupancy_f32(g.bucket, g.exact, g.kind, false, g.threads, g.smem, !g.uniform, false, g.wide);
     if (g.occ_many < 1) return fail(VP_ECUDA, "sampling kernel cannot be resident (smem %zu)", g.smem);
     g.blocks = n_sm * std::min(g.occ_many, 2);
     set_task(g, expect);
@@ -897,7 +923,7 @@ vp_status vp::launch_group(const Desc *d_desc, Group &g, cudaStream_t stream) {
         a.prm_words = g.prm_words;
         e = g.prec == VP_FP64
                 ? launch_sample_f64(g.bucket, g.exact, g.kind, g.blocks, g.threads, g.smem, stream, a, !g.uniform)
-                : launch_sample_f32(g.bucket, g.exact, g.kind, g.blocks, g.threads, g.smem, stream, a, !g.uniform);
+                : launch_sample_f32(g.bucket, g.exact, g.kind, g.blocks, g.threads, g.smem, stream, a, !g.uniform, g.wide);
     }
     if (e != cudaSuccess) return fail(VP_ECUDA, "sampling launch: %s", cudaGetErrorString(e));
     return VP_OK;
@@ -938,7 +964,7 @@ static vp_status time_group(Set &s, Group &g, cudaStream_t stream, float *best_m
 // shape: kernel (precision, bucket, exactness, kind), histogram size, constants,
 // number of integrals and the order of magnitude of their samples.
 struct TuneKey {
-    int prec, bucket, exact, kind, hist_shared, bins, prm_words, members, dev;
+    int prec, bucket, exact, kind, hist_shared, threads, bins, prm_words, members, dev;
     int log2_samples;
     bool operator==(const TuneKey &o) const { return memcmp(this, &o, sizeof *this) == 0; }
 };
@@ -958,6 +984,7 @@ static TuneKey tune_key(const Set &s, const Group &g, double expect) {
     k.exact = g.exact;
     k.kind = g.kind;
     k.hist_shared = g.hist_shared * 4 + g.hist_one;
+    k.threads = g.threads;
     k.bins = g.hist_words;
     k.prm_words = g.prm_words;
     k.members = (int)g.members.size();

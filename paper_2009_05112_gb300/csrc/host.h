@@ -99,6 +99,7 @@ struct Group {
     uint32_t task = 0;
     size_t smem = 0;
     bool one = false;  // a single integral: the cluster kernel with constants in parameters
+    bool wide = false;    // the task kernel's wide CTA (kWideThreads)
     bool uniform = true;  // every member has the same strata on every axis (else: one only)
     bool mo = false;      // several outputs (App. B): the FP64 one-integral kernel that sums them
     bool solo = false;    // a group of one member by construction (several outputs)

@@ -12,6 +12,9 @@ cudaError_t launch_eval_f32_g(int bucket, int kind, cudaStream_t s, const Desc *
 const void *kptr_one_f32_x(int bucket, int kind);
 const void *kptr_one_f32_p1(int bucket, int kind);
 const void *kptr_many_f32_x(int bucket, int kind);
+const void *kptr_many_f32_wg(int bucket, int kind);
+const void *kptr_many_f32_wx(int bucket, int kind);
+const void *kptr_many_f32_wax(int bucket, int kind);
 cudaError_t launch_eval_f32_x(int bucket, int kind, cudaStream_t s, const Desc *desc, int member, int64_t n, const uint64_t *h, const uint32_t *j, uint32_t t, double *x, int32_t *idx, double *jac, double *f, int pw);
 const void *kptr_one_f64_g(int bucket, int kind);
 const void *kptr_one_f64_mo(int bucket, int kind);
@@ -20,9 +23,13 @@ const void *kptr_many_f64_ax(int bucket, int kind);
 const void *kptr_many_f64_g(int bucket, int kind);
 cudaError_t launch_eval_f64_g(int bucket, int kind, cudaStream_t s, const Desc *desc, int member, int64_t n, const uint64_t *h, const uint32_t *j, uint32_t t, double *x, int32_t *idx, double *jac, double *f, int pw);
 
-// (p1: the one-integral FP32 kernel's single-peak form, dimension-exact buckets)
+// (p1: the one-integral FP32 kernel's single-peak form, dimension-exact buckets;
+// wide: the FP32 task kernel's CTA of kWideThreads)
 static const void *pick(bool f64, int bucket, bool exact, int kind, bool one, bool mo = false,
-                        bool ax = false, bool p1 = false) {
+                        bool ax = false, bool p1 = false, bool wide = false) {
+    if (wide)
+        return ax ? kptr_many_f32_wax(bucket, kind)
+                  : (exact ? kptr_many_f32_wx(bucket, kind) : kptr_many_f32_wg(bucket, kind));
     if (f64 && one && mo) return kptr_one_f64_mo(bucket, kind);
     if (!f64 && one && exact && p1 && kind != VP_POSTERIOR) return kptr_one_f32_p1(bucket, kind);
     if (!one && ax) return f64 ? kptr_many_f64_ax(bucket, kind) : kptr_many_f32_ax(bucket, kind);
@@ -32,8 +39,9 @@ static const void *pick(bool f64, int bucket, bool exact, int kind, bool one, bo
 }
 
 static cudaError_t launch_many(bool f64, int bucket, bool exact, int kind, dim3 grid, dim3 block,
-                               size_t smem, cudaStream_t s, const SampleArgs &a, bool ax) {
-    const void *k = pick(f64, bucket, exact, kind, false, false, ax);
+                               size_t smem, cudaStream_t s, const SampleArgs &a, bool ax,
+                               bool wide = false) {
+    const void *k = pick(f64, bucket, exact, kind, false, false, ax, false, wide);
     if (!k) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -73,8 +81,8 @@ static cudaError_t launch_one(bool f64, int bucket, bool exact, int kind, dim3 g
 }
 
 cudaError_t launch_sample_f32(int bucket, bool exact, int kind, dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t s, const SampleArgs &a, bool ax) {
-    return launch_many(false, bucket, exact, kind, grid, block, smem, s, a, ax);
+                              cudaStream_t s, const SampleArgs &a, bool ax, bool wide) {
+    return launch_many(false, bucket, exact, kind, grid, block, smem, s, a, ax, wide);
 }
 cudaError_t launch_sample_f64(int bucket, bool exact, int kind, dim3 grid, dim3 block, size_t smem,
                               cudaStream_t s, const SampleArgs &a, bool ax) {
@@ -100,8 +108,9 @@ struct SmemLimit {
 static std::vector<SmemLimit> g_smem_limit;
 
 static cudaError_t smem_config(bool f64, int bucket, bool exact, int kind, bool one, int max_smem,
-                               bool mo = false, bool ax = false, bool p1 = false) {
-    const void *k = pick(f64, bucket, exact, kind, one, mo, ax, p1);
+                               bool mo = false, bool ax = false, bool p1 = false,
+                               bool wide = false) {
+    const void *k = pick(f64, bucket, exact, kind, one, mo, ax, p1, wide);
     if (!k) return cudaErrorInvalidValue;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -120,8 +129,8 @@ static cudaError_t smem_config(bool f64, int bucket, bool exact, int kind, bool 
     return cudaSuccess;
 }
 cudaError_t sample_smem_config_f32(int bucket, bool exact, int kind, bool one, int max_smem,
-                                   bool ax, bool p1) {
-    return smem_config(false, bucket, exact, kind, one, max_smem, false, ax, p1);
+                                   bool ax, bool p1, bool wide) {
+    return smem_config(false, bucket, exact, kind, one, max_smem, false, ax, p1, wide);
 }
 cudaError_t sample_smem_config_f64(int bucket, bool exact, int kind, bool one, int max_smem,
                                    bool mo, bool ax) {
@@ -129,16 +138,16 @@ cudaError_t sample_smem_config_f64(int bucket, bool exact, int kind, bool one, i
 }
 
 static int occupancy(bool f64, int bucket, bool exact, int kind, bool one, int threads, size_t smem,
-                     bool mo = false, bool ax = false, bool p1 = false) {
-    const void *k = pick(f64, bucket, exact, kind, one, mo, ax, p1);
+                     bool mo = false, bool ax = false, bool p1 = false, bool wide = false) {
+    const void *k = pick(f64, bucket, exact, kind, one, mo, ax, p1, wide);
     int n = 0;
     if (!k || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess)
         return 0;
     return n;
 }
 int sample_occupancy_f32(int bucket, bool exact, int kind, bool one, int threads, size_t smem,
-                         bool ax, bool p1) {
-    return occupancy(false, bucket, exact, kind, one, threads, smem, false, ax, p1);
+                         bool ax, bool p1, bool wide) {
+    return occupancy(false, bucket, exact, kind, one, threads, smem, false, ax, p1, wide);
 }
 int sample_occupancy_f64(int bucket, bool exact, int kind, bool one, int threads, size_t smem,
                          bool mo, bool ax) {

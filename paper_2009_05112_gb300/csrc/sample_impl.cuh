@@ -39,6 +39,8 @@ namespace vp {
 constexpr int kHistGlobal = 0, kHistShared = 1, kHistCompact = 2;
 // dynamic shared memory the one-integral kernel may use (one CTA per SM)
 constexpr size_t kOneSmemMax = 220 * 1024;
+// ... and the task kernel's two CTAs per SM, each
+constexpr size_t kTwoSmemMax = 112 * 1024;
 
 // Launch arguments when the launch serves several integrals (tasks).
 struct SampleArgs {
@@ -1569,17 +1571,15 @@ __global__ void __launch_bounds__(one_max_threads(DMAX, F64, P1), 1)
 // first) and its warps pull warp chunks of the task from a shared counter; the
 // CTA's histograms are flushed when it moves to another integral.
 // Bound: latency.  What limits it is warps per SM, hence registers: the
-// integral's constants, pointers and round keys live in shared memory, the
-// sample loop is compiled for the integral's own dimension, and the FP32 peaks
-// up to D = 12 take one CTA of 768 threads per SM.  512 integrals of 2 to 12
-// dimensions (N_ev 1e4 to 1e6, 15 iterations): 169 ms with everything in
-// registers, two CTAs of 256 (spilling) and one guarded loop; 155 with shared
-// constants; 141 with 768 threads; 124 with a loop per dimension (129 with
-// 1024 threads).
+// integral's constants, pointers and round keys live in shared memory (two CTAs
+// of 256 read them into registers where those suffice, see kInRegs), and large
+// sets of FP32 peaks up to D = 12 take one CTA of 768 threads per SM whose
+// sample loop is compiled for the integral's own dimension.  512
+// integrals of 2 to 12 dimensions (N_ev 1e4 to 1e6, 15 iterations): 169 ms with
+// everything in registers, two CTAs of 256 (spilling) and one guarded loop; 155
+// with shared constants; 141 with 768 threads; 124 with a loop per dimension
+// (129 with 1024 threads).
 // ---------------------------------------------------------------------------
-// (AX: the strata per axis from each integral's descriptor, for sets with
-// integrals whose strata differ between axes, §3.2; a separate instantiation
-// so that the other sets keep the one count in registers)
 // The sample loop for the member's own dimension, one instantiation per D up
 // to DMAX (the same operations as the guarded loop, which tests every axis up
 // to DMAX against the dimension).
@@ -1596,17 +1596,28 @@ __device__ __forceinline__ void run_of_dim(const LoopS &L, const Ptrs &P, const 
         run_of_dim<D + 1, DMAX, KIND>(L, P, prm, s0, s1, h, lo_off, hi_off, hs, hs_t, hc, sexp);
 }
 
-// Largest CTA of the task kernel, which sets its registers: 768 threads (80
-// registers) for the FP32 peaks up to D = 12, else 256 twice (128 registers).
-__host__ __device__ constexpr int many_max_threads(int dmax, bool f64, int kind) {
-    return !f64 && kind != VP_POSTERIOR && dmax <= 12 ? 768 : 256;
+// The task kernel's two CTAs, which set its registers: 256 threads, two per SM
+// (128 registers), or, wide, one of 768 threads (80 registers; FP32 peaks up to
+// D = 12, histograms in shared memory: see group_config_many for when).
+constexpr int kWideThreads = 768;
+__host__ __device__ constexpr bool many_wide(int dmax, bool f64, int kind) {
+    return !f64 && kind != VP_POSTERIOR && dmax <= 12;
 }
 
-template <int DMAX, bool EXACT, bool F64, int KIND, bool AX = false>
-__global__ void __launch_bounds__(many_max_threads(DMAX, F64, KIND), many_max_threads(DMAX, F64, KIND) > 256 ? 1 : 2)
+// (AX: the strata per axis from each integral's descriptor, for sets with
+// integrals whose strata differ between axes, §3.2; a separate instantiation
+// so that the other sets read the one count)
+template <int DMAX, bool EXACT, bool F64, int KIND, bool AX = false, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? kWideThreads : 256, WIDE ? 1 : 2)
     k_sample_many(SampleArgs a) {
+    static_assert(!WIDE || many_wide(DMAX, F64, KIND), "wide form");
     typedef typename Real<F64>::T T;
-    constexpr bool kOwnDim = many_max_threads(DMAX, F64, KIND) > 256 && !EXACT && !AX;
+    constexpr bool kOwnDim = WIDE && !EXACT && !AX;
+    // with 128 registers and FP32 the constants are read into registers once a
+    // task: in a short task the latency of reading them again shows (a step of
+    // two 20-D integrals of 2e4 samples 117 -> 82 us, two of 3-D at 3e6 369 ->
+    // 359); not larger posteriors, whose points need the registers
+    constexpr bool kInRegs = !WIDE && !F64 && (KIND != VP_POSTERIOR || DMAX <= 8);
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_task, s_wc;
     __shared__ uint4 s_keys[5];
@@ -1715,6 +1726,20 @@ __global__ void __launch_bounds__(many_max_threads(DMAX, F64, KIND), many_max_th
         const uint64_t t0 = (task - __ldg(a.chunk_base + g)) * (uint64_t)a.task;
         const uint64_t t1 = min(t0 + (uint64_t)a.task, P.n_total);
         const uint32_t n_wc = ((uint32_t)(t1 - t0) + wchunk - 1) / wchunk;  // 32-bit (no FP64 units)
+        Loop Lr;
+        Ptrs Pr;
+        if constexpr (kInRegs) {
+            Pr = P;
+            *(LoopBase *)&Lr = L;
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const uint4 k = s_keys[i];
+                Lr.rk0[2 * i] = k.x;
+                Lr.rk1[2 * i] = k.y;
+                Lr.rk0[2 * i + 1] = k.z;
+                Lr.rk1[2 * i + 1] = k.w;
+            }
+        }
         for (;;) {
             uint32_t c = 0;
             if (lane == 0) c = atomicAdd(&s_wc, 1u);
@@ -1728,10 +1753,13 @@ __global__ void __launch_bounds__(many_max_threads(DMAX, F64, KIND), many_max_th
             const uint64_t h =
                 lane_find_hcube(P.off, P.n_hc, hb, s0, s0 < s1, lane, &lo_off, &hi_off);
             if (s0 < s1) {
-                if (kOwnDim && a.hist_shared) {
-                    if constexpr (kOwnDim)
-                        run_of_dim<1, DMAX, KIND>(L, P, s_prm, s0, s1, h, lo_off, hi_off, hs, hs_t,
-                                                  hc, s_sexp);
+                if constexpr (kOwnDim) {  // (wide: the histograms are shared)
+                    run_of_dim<1, DMAX, KIND>(L, P, s_prm, s0, s1, h, lo_off, hi_off, hs, hs_t, hc,
+                                              s_sexp);
+                } else if constexpr (kInRegs) {
+                    run_samples<DMAX, EXACT, F64, KIND, false, AX>(
+                        Lr, s_strata, Pr, s_prm, s0, s1, h, lo_off, hi_off, hs, hs_t, hc,
+                        a.hist_shared ? kHistShared : kHistGlobal, s_sexp);
                 } else {
                     run_samples<DMAX, EXACT, F64, KIND, false, AX>(
                         L, s_strata, P, s_prm, s0, s1, h, lo_off, hi_off, hs, hs_t, hc,
@@ -1870,9 +1898,11 @@ __host__ __device__ constexpr int bucket_dim(int b) {
     return b == 0 ? 4 : b == 1 ? 8 : b == 2 ? 12 : b == 3 ? 16 : b == 4 ? 20 : 24;
 }
 // Several integrals (tasks) / one integral (cluster launch of cs CTAs per cluster).
-// (ax: the task kernel with the strata per axis from the descriptors, §3.2)
+// (ax: the task kernel with the strata per axis from the descriptors, §3.2;
+// wide: its CTA of kWideThreads)
 cudaError_t launch_sample_f32(int bucket, bool exact, int kind, dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t s, const SampleArgs &a, bool ax = false);
+                              cudaStream_t s, const SampleArgs &a, bool ax = false,
+                              bool wide = false);
 cudaError_t launch_sample_f64(int bucket, bool exact, int kind, dim3 grid, dim3 block, size_t smem,
                               cudaStream_t s, const SampleArgs &a, bool ax = false);
 cudaError_t launch_sample_one_f32(int bucket, bool exact, int kind, dim3 grid, dim3 block,
@@ -1888,7 +1918,7 @@ cudaError_t launch_eval_f64(int bucket, bool exact, int kind, cudaStream_t s, co
 // (p1: the one-integral kernel's single-peak form, chosen at launch when the
 // FP32 integrand has one peak and the bucket is dimension-exact)
 cudaError_t sample_smem_config_f32(int bucket, bool exact, int kind, bool one, int max_smem,
-                                   bool ax = false, bool p1 = false);
+                                   bool ax = false, bool p1 = false, bool wide = false);
 // §4.2: the data histogram of the map's training (buffer buf; f NULL: the integrand).
 cudaError_t launch_precondition(int bucket, int kind, cudaStream_t s, const Desc *desc, int member,
                                 int64_t n, const double *x, const double *f, uint32_t buf);
@@ -1896,7 +1926,7 @@ cudaError_t launch_precondition(int bucket, int kind, cudaStream_t s, const Desc
 cudaError_t sample_smem_config_f64(int bucket, bool exact, int kind, bool one, int max_smem,
                                    bool mo = false, bool ax = false);
 int sample_occupancy_f32(int bucket, bool exact, int kind, bool one, int threads, size_t smem,
-                         bool ax = false, bool p1 = false);
+                         bool ax = false, bool p1 = false, bool wide = false);
 int sample_occupancy_f64(int bucket, bool exact, int kind, bool one, int threads, size_t smem,
                          bool mo = false, bool ax = false);
 // Resident CTAs of the one-integral kernel with clusters of cs CTAs (0 if it cannot run).

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(256) ks_sum(const double *d_h, uint64_t n_hc, 
     double S[1];  // the block sums in the library's fixed tree order
     vp::block_tree_sum<1>(sc->part, gridDim.x, sh, S);
     if (t != 0) return;
+    sc->done_sum = 0u;  // (for the next call, should a later launch of this one fail)
     sc->sum_d = S[0];
     // (c only where sum d and the quotient are normal numbers and no N_ev d_h
     // can overflow, so that alloc_one's product is within a few ulp of the
@@ -209,14 +210,20 @@ __global__ void __launch_bounds__(256) ks_alloc(const double *d_h, uint64_t n_hc
         const unsigned q = threadIdx.x * kV + k;
         if (q < gridDim.x) sc->bsum[q] = ex + v[k];
     }
-    if (threadIdx.x == 0) off[n_hc] = tot;
+    if (threadIdx.x == 0) {
+        off[n_hc] = tot;
+        sc->done_alloc = 0u;  // (see done_sum)
+    }
 }
 
 template <bool VEC>
 __global__ void __launch_bounds__(256) ks_offsets(const uint32_t *n_h, uint64_t n_hc,
-                                                  uint64_t *off, const StaticScratch *sc) {
+                                                  uint64_t *off, StaticScratch *sc) {
     __shared__ unsigned long long s_w[8];
     vp::pdl_wait();
+    // (whatever overlapping calls may have left: the last of their calls to get
+    // here leaves zeros, every kernel of theirs that counts being done)
+    if (blockIdx.x == 0 && threadIdx.x == 0) sc->done_sum = sc->done_alloc = 0u;
     if (!vp::finite_bits(__ldcg(&sc->sum_d))) return;
     const uint64_t h0 = (uint64_t)blockIdx.x * 1024 + 4u * threadIdx.x;
     const bool full = h0 + 4 <= n_hc;
@@ -312,18 +319,13 @@ extern "C" vp_status vp_alloc_static(const double *d_h, int64_t n_hc, int64_t n_
     cudaStream_t s = (cudaStream_t)stream;
     const unsigned blocks = (unsigned)(((uint64_t)n_hc + 1023) / 1024);
     const bool vec = (((uintptr_t)d_h | (uintptr_t)n_h | (uintptr_t)offsets) & 15u) == 0;
-    // the two last-block counters start at zero whatever an earlier call left
-    // (one whose later launches failed, or calls that overlapped)
-    cudaError_t e = cudaMemsetAsync(&sc->done_sum, 0, 2 * sizeof(unsigned int), s);
-    if (e == cudaSuccess)
-        e = launch256(ks_sum, blocks, s, d_h, (uint64_t)n_hc, (double)n_ev, sc);
+    cudaError_t e = launch256(ks_sum, blocks, s, d_h, (uint64_t)n_hc, (double)n_ev, sc);
     if (e == cudaSuccess)
         e = launch256(vec ? ks_alloc<true> : ks_alloc<false>, blocks, s, d_h, (uint64_t)n_hc,
                       (double)n_ev, plus2 ? 1 : 0, n_h, offsets, sc);
     if (e == cudaSuccess)
         e = launch256(vec ? ks_offsets<true> : ks_offsets<false>, blocks, s,
-                      (const uint32_t *)n_h, (uint64_t)n_hc, offsets,
-                      (const StaticScratch *)sc);
+                      (const uint32_t *)n_h, (uint64_t)n_hc, offsets, sc);
     if (e != cudaSuccess) {
         vp::set_error_message(VP_ECUDA, cudaGetErrorString(e));
         return VP_ECUDA;

@@ -523,12 +523,13 @@ static vp_status plan_groups(Set &s) {
 // a step, two CTAs / one wide: 80 / 97 us at 3e4 samples each, 161 / 174 at
 // 1e5, 416 / 305 at 3e5; 4 of 8-D at 1e5: 56 / 74).  Strata per axis, whose
 // loop is not compiled per dimension: from twice that (32 of 5 to 8 dimensions
-// at 1e5: 262 / 291; at 3e5 647 / 585).  Histograms that only one CTA per SM
-// can hold, added in global memory otherwise: from half of it (2 of 12-D,
-// N_g = 1000, at 1e6: 392 / 184).  At most a quarter of the samples on one or
-// two axes, where 24 warps add to few bins of one histogram (4 of 2-D at 3e6:
-// 1210 / 1620), and up to D = 4 four integrals or more (2 of 3-D at 1e6: 145 /
-// 160; 16 at 3e5: 289 / 244).
+// at 1e5: 262 / 291; at 3e5 647 / 585), and so up to D = 4 (32 of 4-D at 1e5:
+// 210 / 219; 16 at 3e5 278 / 241).  Histograms that only one CTA per SM can
+// hold, added in global memory otherwise: from half of it (2 of 12-D, N_g =
+// 1000, at 1e6: 392 / 184).  At most a quarter of the samples on one or two
+// axes, where 24 warps add to few bins of one histogram (4 of 2-D at 3e6: 1210 /
+// 1620), and up to D = 4 four integrals or more (2 of 3-D at 1e6: 145 / 160; 16
+// at 3e5: 289 / 244).
 constexpr double kWideMinSamples = 2.5e6;
 static bool wide_pays(const std::vector<const Member *> &m, const Group &g, double expect,
                       size_t hist_bytes, size_t prm_bytes) {
@@ -541,7 +542,7 @@ static bool wide_pays(const std::vector<const Member *> &m, const Group &g, doub
         if (m[i]->p.dim <= 2) low += (double)m[i]->p.n_ev + 2.0 * (double)m[i]->n_hc;
     if (low > 0.25 * expect) return false;
     if (hist_bytes + prm_bytes > kTwoSmemMax) return expect >= 0.5 * kWideMinSamples;
-    return expect >= (g.uniform ? 1.0 : 2.0) * kWideMinSamples;
+    return expect >= (g.uniform && bucket_dim(g.bucket) > 4 ? 1.0 : 2.0) * kWideMinSamples;
 }
 
 // Task-kernel launch shape of a group: the wide CTA where it pays, else two CTAs

@@ -1547,9 +1547,12 @@ static vp_status shard_check(vp_ctx *c) {
 
 // Launch shape of a part of an FP32 integral with shared-memory histograms, by
 // rule: a CTA adds its d_i terms in FP32 and a cluster its CTAs' sums, so the
-// shape decides the roundings of the exported sums (16-D, 250,000 samples: 1e-9
-// to 3e-9 of their norm between shapes, a few 1e-10 between runs of one), and a
-// shape picked by a stopwatch would let two runs, or two ranks, differ by them.
+// shape decides the roundings of the exported sums, and a shape picked by a
+// stopwatch would let two runs, or two ranks, differ by them.  (16-D, 250,000
+// samples in 4 parts, relative to their norm: clusters of 1 against 2 differ by
+// 2.7e-9 .. 3.2e-9 in the first iteration and 6e-9 .. 7.6e-9 in the second; what
+// is left is the order of a bin's adds, between runs of one shape 1e-10 ..
+// 1.8e-9 and 2.1e-9 .. 3.7e-9.)
 // Pairs of CTAs (half the global reductions of a flush), one CTA of the
 // kernel's largest size per SM.  Peaks up to D = 8: the largest size that gives
 // every lane a sample (7-D, 3e5 samples in 4 parts: 512 threads 100 us, 1024

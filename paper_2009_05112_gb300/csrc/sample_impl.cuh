@@ -1172,8 +1172,8 @@ __device__ __forceinline__ void run_samples_t(const LT &L, const Strata *S, cons
             } else {
                 float x[DMAX];
                 int fe;
-                point32<DMAX, EXACT, KIND, KP, AX, kShort>(L, S, (const float *)prm, (uint32_t)h, j, kc, x,
-                                                   idx, Jm, Je, f, fe);
+                point32<DMAX, EXACT, KIND, KP, AX, kShort>(L, S, (const float *)prm, (uint32_t)h, j,
+                                                           kc, x, idx, Jm, Je, f, fe);
                 Je += fe;  // J f = (Jm f) 2^(Je + fe)
             }
             float jf = Jm * f;  // Jm in [1, 2); the last multiply-add of f may leave it subnormal
@@ -1462,9 +1462,10 @@ __global__ void __launch_bounds__(one_max_threads(DMAX, F64, P1), 1)
         // warp at work, and the FP64 path, whose warp instructions cost the
         // same whatever their lanes do, paid for all 32.  (FP64 up to 8 samples
         // per lane: beyond it the idle lanes cost less than a warp in nine.
-        // FP32 at one per lane, up to D = 8 and not in parts: its sums depend on
-        // which samples a lane, a warp's combine and a CTA's histogram add.  A 4-D
-        // FP64 job of 1e4 samples: 1104 -> 940 us.)
+        // FP32 at one per lane and up to D = 8 only, where every lane's sample goes
+        // to its hypercube's FP64 sums by itself whatever the split; its
+        // histograms' FP32 sums are regrouped, so not in parts, which export
+        // them.  A 4-D FP64 job of 1e4 samples: 1104 -> 940 us.)
         uint32_t Ws = W, ws = w;
         if constexpr (F64 || DMAX <= 8) {
             const uint32_t rounds = n_st / (32u * W) + (n_st % (32u * W) != 0u ? 1u : 0u);
@@ -1574,11 +1575,11 @@ __global__ void __launch_bounds__(one_max_threads(DMAX, F64, P1), 1)
 // integral's constants, pointers and round keys live in shared memory (two CTAs
 // of 256 read them into registers where those suffice, see kInRegs), and large
 // sets of FP32 peaks up to D = 12 take one CTA of 768 threads per SM whose
-// sample loop is compiled for the integral's own dimension.  512
-// integrals of 2 to 12 dimensions (N_ev 1e4 to 1e6, 15 iterations): 169 ms with
-// everything in registers, two CTAs of 256 (spilling) and one guarded loop; 155
-// with shared constants; 141 with 768 threads; 124 with a loop per dimension
-// (129 with 1024 threads).
+// sample loop is compiled for the integral's own dimension.  512 integrals of 2
+// to 12 dimensions (N_ev 1e4 to 1e6, 15 iterations): 169 ms with everything in
+// registers, two CTAs of 256 (spilling) and one guarded loop; 155 with shared
+// constants; 141 with 768 threads; 124 with a loop per dimension (129 with 1024
+// threads).
 // ---------------------------------------------------------------------------
 // The sample loop for the member's own dimension, one instantiation per D up
 // to DMAX (the same operations as the guarded loop, which tests every axis up
@@ -1809,8 +1810,8 @@ __global__ void k_eval(const Desc *desc, int member, int64_t n, const uint64_t *
             hcube_offsets<DMAX, true>(L, S, kd, kc);
             int fe;
             Idx<DMAX, false> ix;
-            point32<DMAX, EXACT, KIND, false, true, false>(L, S, sprm, (uint32_t)hs[k], js[k], kc, x, ix,
-                                                    Jm, Je, ff, fe);
+            point32<DMAX, EXACT, KIND, false, true, false>(L, S, sprm, (uint32_t)hs[k], js[k], kc,
+                                                           x, ix, Jm, Je, ff, fe);
 #pragma unroll
             for (int mu = 0; mu < DMAX; ++mu) idx[mu] = mu < dim ? ix.get(mu) : 0;
 #pragma unroll
